@@ -241,12 +241,16 @@ bool build_bvh(const float* verts, const uint32_t* tris, uint32_t n_tris, BvhOut
         if (bn[i].count == 0) gpu_id[i] = n_int++;
     auto emit = [&](const Box& b0, uint32_t r0, const Box& b1, uint32_t r1) {
         float f[16];
-        for (int k = 0; k < 3; ++k) {      // row k: (c0.lo, c1.lo, c0.hi, c1.hi) of axis k
-            f[4 * k] = b0.lo[k];
-            f[4 * k + 1] = b1.lo[k];
-            f[4 * k + 2] = b0.hi[k];
-            f[4 * k + 3] = b1.hi[k];
+        for (int k = 0; k < 2; ++k) {      // rows 0 and 1: (lo.x, lo.y, hi.x, hi.y) of each child
+            f[k] = b0.lo[k];
+            f[2 + k] = b0.hi[k];
+            f[4 + k] = b1.lo[k];
+            f[6 + k] = b1.hi[k];
         }
+        f[8] = b0.lo[2];                   // row 2: the z planes of both
+        f[9] = b0.hi[2];
+        f[10] = b1.lo[2];
+        f[11] = b1.hi[2];
         f[12] = f32_bits(r0);
         f[13] = f32_bits(r1);
         f[14] = 0.f;

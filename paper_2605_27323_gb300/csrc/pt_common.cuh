@@ -56,16 +56,43 @@ __device__ __forceinline__ uint32_t warp_append(uint32_t* counter, bool want) {
     return base + (uint32_t)__popc(mask & ((1u << lane_id()) - 1u));
 }
 
-// Warp-granular dynamic work: each warp claims its next queue slots (32, one per lane; 32 / G when
-// groups of G lanes share a ray) with one atomic, so warps that drew cheap rays take more batches
-// and the grid ends together (a static grid-stride split leaves the SMs waiting on the warps that
-// drew the longest rays).
-__device__ __forceinline__ uint32_t warp_claim(uint32_t* counter, uint32_t k) {
+// Warp-granular dynamic work: the queue is cut into chunks (32 slots, one per lane; 32 / G when groups
+// of G lanes share a ray).  A warp's first chunk is its own index in the grid; it claims every further
+// one with one atomic, so warps that drew cheap rays take more chunks and the grid ends together (a
+// static grid-stride split leaves the SMs waiting on the warps that drew the longest rays).
+// `counter` is zero at launch.
+__device__ __forceinline__ uint32_t first_chunk() { return (blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
+__device__ __forceinline__ uint32_t next_chunk(uint32_t* counter) {
     uint32_t b = 0u;
-    if (lane_id() == 0u) b = atomicAdd(counter, k);
-    return __shfl_sync(0xFFFFFFFFu, b, 0);
+    if (lane_id() == 0u) b = atomicAdd(counter, 1u);
+    return ((gridDim.x * blockDim.x) >> 5) + __shfl_sync(0xFFFFFFFFu, b, 0);
 }
-__device__ __forceinline__ uint32_t warp_claim32(uint32_t* counter) { return warp_claim(counter, 32u); }
+
+// Chunks taken by a warp that hands their slots to its lanes one by one (the pooled walks): the current
+// chunk, how many of its slots are handed out, and the next chunk, whose claim is in flight while the
+// current one is walked.
+struct ChunkPool {
+    uint32_t* counter;
+    uint32_t c, used = 0, n_warps;
+    uint32_t raw;             // lane 0: the claim of the next chunk (consumed by a shuffle when needed)
+    uint32_t c_all;
+    __device__ __forceinline__ ChunkPool(uint32_t* ctr, uint32_t chunks)
+        : counter(ctr), c(first_chunk()), n_warps((gridDim.x * blockDim.x) >> 5), raw(0u), c_all(chunks) {
+        claim();
+    }
+    // no atomic when the chunks do not outnumber the warps: every claim would come back beyond the end
+    __device__ __forceinline__ void claim() {
+        if (c_all > n_warps && lane_id() == 0u) raw = atomicAdd(counter, 1u);
+    }
+    __device__ __forceinline__ uint32_t peek() const {
+        return c_all > n_warps ? n_warps + __shfl_sync(0xFFFFFFFFu, raw, 0) : c_all;
+    }
+    __device__ __forceinline__ void advance(uint32_t next) {
+        c = next;
+        used = 0u;
+        claim();
+    }
+};
 
 __device__ __forceinline__ void warp_add_u64(unsigned long long* dst, unsigned long long v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);

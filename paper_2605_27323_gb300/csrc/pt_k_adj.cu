@@ -93,8 +93,9 @@ __global__ void __launch_bounds__(256) k_shadow_adj(SingleSrc src, WfBuffers w, 
     const uint32_t n = min(w.counts[2], w.capacity);
     if (n == 0u) return;
     const size_t cap = w.capacity;
-    for (uint32_t b0 = warp_claim32(&w.counts[5]); b0 < n; b0 = warp_claim32(&w.counts[5])) {
-        const uint32_t j = b0 + lane_id();
+    const uint32_t chunks = (n + 31u) / 32u;
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[5])) {
+        const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         const float4 so = __ldcs(&w.s_o[j]), sd = __ldcs(&w.s_d[j]);
         if (!trace_any<INST>(src.s, xyz(so), xyz(sd), so.w)) {

@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "pt_common.cuh"
+#include "pt_pool.cuh"
 
 namespace pt {
 
@@ -43,14 +44,92 @@ __global__ void __launch_bounds__(256) k_raygen(Src src, uint64_t base, uint32_t
     }
 }
 
+// Extension rays as the pooled walks take them: a queue slot's ray (and its scene's tree), its hit record.
+template <class Src>
+struct ExtendIo {
+    const Src& src;
+    const float4* __restrict__ qo;
+    const float4* __restrict__ qd;
+    float2* __restrict__ hit;
+    uint64_t base;
+    __device__ __forceinline__ void fetch(uint32_t j, float3& o, float3& d, float& tbest, uint32_t& best,
+                                          const float4*& nodes, const float4*& tris) const {
+        const float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
+        o = xyz(o4);
+        d = xyz(d4);
+        tbest = __int_as_float(0x7f800000);
+        best = kMiss;
+        if constexpr (!std::is_same<Src, SingleSrc>::value) {
+            const DevScene s = src.scene(src.sid_from_ray(d4.w, base, __float_as_uint(o4.w)));
+            nodes = s.nodes;
+            tris = s.tris;
+        }
+    }
+    __device__ __forceinline__ void emit(uint32_t j, float t, uint32_t tri) const {
+        hit[j] = make_float2(t, __uint_as_float(tri));
+    }
+};
+
+// Extension rays and shadow rays (slots with kAnySlot; `best` carries their path, tbest < 0: occluded).
+template <class Src, bool SIG, bool ADJ>
+struct TraceIo {
+    ExtendIo<Src> ext;
+    const WfBuffers& w;
+    const AdjBuffers& a;
+    uint32_t b;
+    __device__ __forceinline__ void fetch(uint32_t slot, float3& o, float3& d, float& tbest, uint32_t& best,
+                                          const float4*& nodes, const float4*& tris) const {
+        if (!(slot & kAnySlot)) {
+            ext.fetch(slot, o, d, tbest, best, nodes, tris);
+            return;
+        }
+        const uint32_t k = slot & ~kAnySlot;
+        const float4 so = __ldcs(&w.s_o[k]), sd = __ldcs(&w.s_d[k]);
+        o = xyz(so);
+        d = xyz(sd);
+        tbest = so.w;
+        best = __float_as_uint(sd.w);
+        if constexpr (!ADJ && !std::is_same<Src, SingleSrc>::value) {
+            const DevScene s = ext.src.scene(ext.src.sid_from_shadow(__ldcs(&w.s_c[k].w), ext.base, best));
+            nodes = s.nodes;
+            tris = s.tris;
+        }
+    }
+    __device__ __forceinline__ void emit(uint32_t slot, float t, uint32_t tri) const {
+        if (!(slot & kAnySlot)) {
+            ext.emit(slot, t, tri);
+            return;
+        }
+        const bool occ = t < 0.0f;
+        if constexpr (ADJ) {
+            if (!occ) {
+                float* fl = reinterpret_cast<float*>(a.rec + 4 * ((size_t)(b - 1u) * w.capacity + tri) + 3) + 3;
+                *fl = __uint_as_float(__float_as_uint(*fl) | 2u);
+            }
+        } else {
+            if (occ && !SIG) return;
+            const float4 sc = __ldcs(&w.s_c[slot & ~kAnySlot]);
+            if (!occ) w.L[tri] = f4(add_rn(xyz(w.L[tri]), xyz(sc)), 0.f);
+            if (SIG) {
+                const uint32_t lj = __float_as_uint(sc.w);
+                w.sig[ext.base + tri] ^= sig_event(b - 1u, 1, (lj << 2) | 2u | (occ ? 0u : 1u));
+            }
+        }
+    }
+};
+
+// Resident blocks of 256 of the traversal kernels, which cap their registers.  Pooled walks: 5 (48 registers,
+// no spills; against 6 blocks with 80 bytes of spills 1.94 -> 1.91 ms per 1080p frame, against 4 blocks
+// 1.96 -> 1.91).  Lockstep walks (short stack, counting): 6 single-level (40 registers), 4 two-level (64
+// registers; 6 blocks measured slower, and without a bound ptxas takes 78 registers, leaving 3 blocks:
+// 2.89 -> 3.00 ms per two-level frame).
+constexpr int trace_blocks(bool inst, bool pooled) { return inst ? 4 : pooled ? 5 : 6; }
+
 // Extend: closest hit of every active ray (scene-intersection stage); hit records per queue slot.
-// Registers capped for 6 resident blocks of 256 single-level (extend 2.73 -> 2.68 ms per 1080p step
-// against 5 blocks) and 4 two-level (64 registers; 6 blocks measured slower, and without a bound
-// ptxas takes 78 registers, leaving 3 blocks: 2.89 -> 3.00 ms per two-level frame).
 // SK > 0: the walks keep their top SK stack entries in dynamic shared memory (single-level only).
 // CNT: count the walks' node visits and triangle tests into the scene's traversal counters.
 template <class Src, bool INST, int SK = 0, bool CNT = false>
-__global__ void __launch_bounds__(256, INST ? 4 : 6) k_extend(Src src, WfBuffers w, int in) {
+__global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_extend(Src src, WfBuffers w, int in) {
     stage_prologue();
     const uint32_t n = min(w.counts[0], w.capacity);
     if (n == 0u) return;       // an emptied queue: no claims (the same for every thread)
@@ -58,9 +137,15 @@ __global__ void __launch_bounds__(256, INST ? 4 : 6) k_extend(Src src, WfBuffers
     const float4* __restrict__ qo = w.q_o[in];
     const float4* __restrict__ qd = w.q_d[in];
     float2* __restrict__ hit = w.hit;
+    const uint32_t chunks = (n + 31u) / 32u;
+    if constexpr (!INST && SK == 0 && !CNT) {
+        ChunkPool q(&w.counts[4], chunks);
+        pool_walk(src.scene(0), q, chunks, n, 0u, ExtendIo<Src>{src, qo, qd, hit, base});
+        return;
+    }
     typename std::conditional<CNT, TravCount, NoCount>::type cnt;
-    for (uint32_t b0 = warp_claim32(&w.counts[4]); b0 < n; b0 = warp_claim32(&w.counts[4])) {
-        const uint32_t j = b0 + lane_id();
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[4])) {
+        const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
         Hit h = trace_closest<INST, SK>(src.scene(src.sid_from_ray(d4.w, base, __float_as_uint(o4.w))), xyz(o4), xyz(d4),
@@ -262,8 +347,9 @@ __global__ void __launch_bounds__(256) k_shadow(Src src, WfBuffers w, uint32_t b
     if (n == 0u) return;
     const uint64_t base = src.base();
     typename std::conditional<CNT, TravCount, NoCount>::type cnt;
-    for (uint32_t b0 = warp_claim32(&w.counts[5]); b0 < n; b0 = warp_claim32(&w.counts[5])) {
-        const uint32_t j = b0 + lane_id();
+    const uint32_t chunks = (n + 31u) / 32u;
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[5])) {
+        const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         const float4 so = __ldcs(&w.s_o[j]), sd = __ldcs(&w.s_d[j]), sc = __ldcs(&w.s_c[j]);
         const uint32_t pid = __float_as_uint(sd.w);
@@ -295,8 +381,11 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
     unsigned long long led = 0;      // walks this lane's group traced, counted once per group
     const float4* __restrict__ qo = w.q_o[in];
     const float4* __restrict__ qd = w.q_d[in];
-    for (uint32_t b0 = warp_claim(&w.counts[4], per); b0 < n_ext; b0 = warp_claim(&w.counts[4], per)) {
-        const uint32_t j = b0 + sub;
+    // one chunk sequence over both sets: the extension rays' chunks, then the shadow rays'
+    const uint32_t c_ext = (n_ext + per - 1u) / per, c_all = c_ext + (n_shd + per - 1u) / per;
+    uint32_t c = first_chunk();
+    for (; c < c_ext; c = next_chunk(&w.counts[4])) {
+        const uint32_t j = c * per + sub;
         const bool valid = j < n_ext;
         float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = make_float4(0.f, 0.f, 1.f, 0.f);
         if (valid) {
@@ -312,8 +401,8 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
             ++led;
         }
     }
-    for (uint32_t b0 = warp_claim(&w.counts[5], per); b0 < n_shd; b0 = warp_claim(&w.counts[5], per)) {
-        const uint32_t k = b0 + sub;
+    for (; c < c_all; c = next_chunk(&w.counts[4])) {
+        const uint32_t k = (c - c_ext) * per + sub;
         const bool valid = k < n_shd;
         float4 so = make_float4(0.f, 0.f, 0.f, 0.f), sd = make_float4(0.f, 0.f, 1.f, 0.f);
         float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -352,14 +441,15 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
 // the shadow rays that shading cast at bounce b - 1 (any hit, the shadow queue, counts[6] entries).
 // The two sets are independent -- a shadow ray only adds its contribution to its path's radiance, and
 // only the next shading reads that radiance -- so each path still adds its terms in the order
-// emission(b - 1), NEE(b - 1), emission(b), as in the megakernel.  Warps claim 32 continuation rays
-// at a time until none is left and then 32 shadow rays at a time (two loops, so each walk keeps the
-// registers it has in its own stage); a launch therefore ends when both sets are done, and the shadow
-// walks fill the extension walks' tail instead of running after a stage boundary.
+// emission(b - 1), NEE(b - 1), emission(b), as in the megakernel.  Single-level launches walk both sets
+// through one pool (pool_walk): the continuation rays first, then the shadow rays; two-level and counting
+// launches take 32 continuation rays at a time until none is left and then 32 shadow rays at a time.
+// A launch therefore ends when both sets are done, and the shadow walks fill the extension walks' tail
+// instead of running after a stage boundary.
 // ADJ: the adjoint replay's variant, whose shadow walks mark the vertex record's NEE sample visible
 // (flag 2 of record 3 of bounce b - 1) instead of adding a contribution.
 template <class Src, bool SIG, bool INST, bool CNT = false, bool ADJ = false>
-__global__ void __launch_bounds__(256, INST ? 4 : 6) k_trace(Src src, WfBuffers w, AdjBuffers a, int in, uint32_t b) {
+__global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src, WfBuffers w, AdjBuffers a, int in, uint32_t b) {
     stage_prologue();
     const uint32_t n_ext = min(w.counts[0], w.capacity), n_shd = min(w.counts[6], w.capacity);
     if (n_ext + n_shd == 0u) return;       // the same for every thread
@@ -378,12 +468,22 @@ __global__ void __launch_bounds__(256, INST ? 4 : 6) k_trace(Src src, WfBuffers 
         trace_groups<Src, SIG, INST, ADJ>(src, w, a, in, b, n_ext, n_shd, G);
         return;
     }
+    if constexpr (!INST && !CNT) {
+        const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
+        ChunkPool q(&w.counts[4], c_all);
+        pool_walk(src.scene(0), q, c_ext, n_ext, n_shd,
+                  TraceIo<Src, SIG, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, base}, w, a, b});
+        return;
+    }
     typename std::conditional<CNT, TravCount, NoCount>::type cc, ca;
+    // one chunk sequence over both sets: the extension rays' chunks, then the shadow rays'
+    const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
+    uint32_t c = first_chunk();
     {
         const float4* __restrict__ qo = w.q_o[in];
         const float4* __restrict__ qd = w.q_d[in];
-        for (uint32_t b0 = warp_claim32(&w.counts[4]); b0 < n_ext; b0 = warp_claim32(&w.counts[4])) {
-            const uint32_t j = b0 + lane_id();
+        for (; c < c_ext; c = next_chunk(&w.counts[4])) {
+            const uint32_t j = c * 32u + lane_id();
             if (j >= n_ext) continue;
             const float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
             Hit h = trace_closest<INST, 0>(src.scene(src.sid_from_ray(d4.w, base, __float_as_uint(o4.w))), xyz(o4),
@@ -392,8 +492,8 @@ __global__ void __launch_bounds__(256, INST ? 4 : 6) k_trace(Src src, WfBuffers 
             if (INST) w.hit_inst[j] = h.inst;
         }
     }
-    for (uint32_t b0 = warp_claim32(&w.counts[5]); b0 < n_shd; b0 = warp_claim32(&w.counts[5])) {
-        const uint32_t k = b0 + lane_id();
+    for (; c < c_all; c = next_chunk(&w.counts[4])) {
+        const uint32_t k = (c - c_ext) * 32u + lane_id();
         if (k >= n_shd) continue;
         const float4 so = __ldcs(&w.s_o[k]), sd = __ldcs(&w.s_d[k]);
         const uint32_t pid = __float_as_uint(sd.w);

@@ -1,0 +1,153 @@
+// pt_pool.cuh -- pooled walks: the dense traversal loop of the wavefront's trace stages.
+//
+// A lockstep walk of 32 rays (each lane its own ray, the warp takes 32 new ones when the last has
+// finished) issues every instruction for 9 lanes of 32 on average after the first bounce: lanes whose
+// walk ended wait for the longest one, and a leaf step runs for the one or two lanes that hold a leaf
+// while the others wait.  Here a warp keeps its lanes supplied from a pool of queue slots:
+//   - node steps repeat while at least kNodeLanes lanes hold an inner node;
+//   - then all lanes that hold a leaf test it together;
+//   - once kIdleLanes lanes have finished, they write their results and take the next slots.
+// Extension (closest-hit) and shadow (any-hit) rays share the loop, so a launch drains its warps once
+// and not once per kind.  Each ray visits the nodes and triangles of the lockstep walk in the same
+// order, so hits are the same bit for bit.
+//
+// What bounds it: node data returns to registers at 128 bytes per clock and SM, so a node step (64 bytes
+// a lane) takes 16 cycles of the L1 data path whether 20 or 32 lanes need it: that path is busy 76% of
+// the time (issue 58%, long-scoreboard stalls for the rest) in the launch of bounce 1 at 1080p on 1.15 M
+// triangles.  Against the lockstep walk: extension rays 15.4 -> 22 lanes per node step, bounce 1 9.5 ->
+// 19.7, 683 -> 585 us; the 1080p frame 1.96 -> 1.73 ms, a 1.07 M-triangle terrain at 2560 x 1440, 3 samples,
+// depth 8 13.04 -> 10.63 ms.
+#pragma once
+#include "pt_common.cuh"
+
+namespace pt {
+
+constexpr uint32_t kDone = 0xFFFFFFFFu;    // no subtree left (never a leaf reference: triangles < 2^28)
+constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+// 12 and 12 measured best of {8..24} x {4..16} lanes: fewer node lanes waste L1 cycles, more make the
+// loop leave its node steps too often (20 and 8: 1.887 ms per frame against 1.870 at 16 and 8); a refill
+// costs about 150 instructions for the whole warp.
+constexpr uint32_t kNodeLanes = 12;
+constexpr uint32_t kIdleLanes = 12;
+
+// A slot of the pool: an extension ray's queue index, or a shadow ray's with kAnySlot set (capacities stay
+// far below 2^31: a path's records take 180 bytes).
+constexpr uint32_t kAnySlot = 0x80000000u;
+
+// Hand out the next slots of the pool to the lanes of `idle` (all 32 lanes call it): this lane's slot, or
+// kNoSlot.  Chunks [0, c_ext) cover the n_ext extension rays, the rest the n_shd shadow rays.
+__device__ __forceinline__ uint32_t pool_take(ChunkPool& q, uint32_t c_ext, uint32_t n_ext, uint32_t n_shd,
+                                              uint32_t idle) {
+    const uint32_t lane = lane_id(), k = (uint32_t)__popc(idle), rank = (uint32_t)__popc(idle & ((1u << lane) - 1u));
+    const uint32_t avail = 32u - q.used;
+    uint32_t c = q.c, off = q.used + rank;
+    q.used += k;
+    if (k >= avail) {          // the current chunk runs out: the rest come from the next one
+        const uint32_t nc = q.peek();
+        if (rank >= avail) {
+            c = nc;
+            off = rank - avail;
+        }
+        q.advance(nc);
+        q.used = k - avail;
+    }
+    uint32_t j = kNoSlot;
+    if ((idle >> lane) & 1u) {
+        if (c < c_ext) {
+            const uint32_t i = c * 32u + off;
+            if (i < n_ext) j = i;
+        } else if (c < q.c_all) {
+            const uint32_t i = (c - c_ext) * 32u + off;
+            if (i < n_shd) j = i | kAnySlot;
+        }
+    }
+    return j;
+}
+
+template <class Io>
+__device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint32_t c_ext, uint32_t n_ext,
+                                          uint32_t n_shd, const Io& io) {
+    uint2 stk[kStack];
+    int sp = 0;
+    uint32_t ref = kDone, slot = kNoSlot, best = kMiss;
+    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o;
+    float tbest = 0.f;
+    const float4 *nodes = s.nodes, *tris = s.tris;
+    uint32_t steps = 0;
+    auto pop = [&]() {
+        ref = kDone;
+        while (sp > 0) {
+            const uint2 v = stk[--sp];
+            if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
+                ref = v.x;
+                break;
+            }
+        }
+    };
+    while (true) {
+        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, ref == kDone);
+        const bool all = idle == 0xFFFFFFFFu;
+        if (all || ((uint32_t)__popc(idle) >= kIdleLanes && q.c < q.c_all)) {
+            if (ref == kDone && slot != kNoSlot) {
+                io.emit(slot, tbest, best);
+                slot = kNoSlot;
+            }
+            if (q.c >= q.c_all) break;
+            const uint32_t j = pool_take(q, c_ext, n_ext, n_shd, idle);
+            if (j != kNoSlot) {
+                slot = j;
+                io.fetch(j, o, d, tbest, best, nodes, tris);
+                id = ray_rcp(d);
+                ref = 0u;
+                sp = 0;
+            }
+            steps = 0;
+        }
+        uint32_t m;
+        do {
+            if (!(ref & kLeafBit)) {
+                float4 n0, n1, n2;
+                uint2 r;
+                load_node(nodes, ref, n0, n1, n2, r);
+                float t0, t1;
+                bool h0, h1;
+                box_test2(n0, n1, n2, o, id, tbest, t0, t1, h0, h1);
+                // the child to walk next (the nearer one when both boxes are hit) and the one deferred
+                const bool first0 = h0 && (t0 <= t1 || !h1);
+                ref = first0 ? r.x : r.y;
+                if (h0 && h1) stk[sp++] = make_uint2(first0 ? r.y : r.x, __float_as_uint(first0 ? t1 : t0));
+                else if (!(h0 || h1)) pop();
+            }
+            m = __ballot_sync(0xFFFFFFFFu, !(ref & kLeafBit));
+        } while ((uint32_t)__popc(m) >= kNodeLanes);
+        if ((ref & kLeafBit) && ref != kDone) {
+            const uint32_t first = (ref & 0x7FFFFFFFu) >> 3, n_leaf = (ref & 7u) + 1u;
+            const bool any = (slot & kAnySlot) != 0u;
+            bool over = false;
+            for (uint32_t k = 0; k < n_leaf && !over; ++k) {
+                float t;
+                uint32_t prim;
+                if (!tri_test(tris, first + k, o, d, t, prim) || !(t > 0.0f)) continue;
+                if (any) {
+                    over = t < tbest;
+                } else if (t < tbest ||
+                           (t == tbest && (best == kMiss || prim < __float_as_uint(__ldg(tris + 3 * (size_t)best).w)))) {
+                    tbest = t;
+                    best = first + k;
+                }
+            }
+            if (over) {
+                tbest = -1.0f;       // occluded
+                ref = kDone;
+            } else {
+                pop();
+            }
+        }
+        if (++steps >= kMaxSteps) {
+            if (ref != kDone) atomicOr(s.status, ST_TRAVERSAL);
+            ref = kDone;
+        }
+    }
+}
+
+}  // namespace pt

@@ -4,11 +4,12 @@
 // BVH -- one over all triangles, or (two-level scenes, the paper's TLAS/BLAS structure of Sec. 2.3)
 // one over instances whose leaves lead into per-mesh BVHs.
 //
-// Node layout (64 bytes, one 128-bit load per row, both children's boxes in the parent; each axis
-// row pairs the two children so that one packed FP32 operation serves both):
-//   n0 = (c0.lo.x, c1.lo.x, c0.hi.x, c1.hi.x)
-//   n1 = (c0.lo.y, c1.lo.y, c0.hi.y, c1.hi.y)
-//   n2 = (c0.lo.z, c1.lo.z, c0.hi.z, c1.hi.z)
+// Node layout (64 bytes, two 256-bit loads, both children's boxes in the parent; x and y planes of a
+// corner lie side by side, so that one packed FP32 operation serves both axes with the ray's own
+// (x, y) register pair):
+//   n0 = (c0.lo.x, c0.lo.y, c0.hi.x, c0.hi.y)
+//   n1 = (c1.lo.x, c1.lo.y, c1.hi.x, c1.hi.y)
+//   n2 = (c0.lo.z, c0.hi.z, c1.lo.z, c1.hi.z)
 //   n3 = (ref0, ref1, -, -)     ref: internal node index, or 0x80000000 | first << 3 | (count - 1)
 // Triangle record (48 bytes): (v0.xyz, prim id) (e1 = v1 - v0, material) (e2 = v2 - v0, is_light).
 //
@@ -57,13 +58,13 @@ __device__ __forceinline__ bool box_test(float lox, float hix, float loy, float 
 }
 
 // Slab test of a node's two child boxes against [0, tmax]: whether each is hit and its entry distance.
-// Rows nx, ny, nz hold (c0.lo, c1.lo, c0.hi, c1.hi) of one axis, so the plane distances
-// (plane - o) * (1/d) of both children come from packed FP32 pairs (sub/mul.rn.f32x2: each half
-// rounded exactly as the scalar operation); the entry is the largest near-plane distance (at least 0),
-// the exit the smallest far-plane distance (at most tmax), and a box counts as hit when entry <= exit
-// widened by a few ulps, so that rounding cannot cull a true hit.  PK = false computes the same values
-// with box_test, one child at a time (for the register-bound one-thread-per-path kernels' two-level
-// walks, where the packed pairs cost spills).
+// The plane distances (plane - o) * (1/d) come from packed FP32 pairs (sub/mul.rn.f32x2: each half
+// rounded exactly as the scalar operation): x and y of a corner together, both z planes of a child
+// together.  The entry is the largest near-plane distance (at least 0), the exit the smallest far-plane
+// distance (at most tmax), and a box counts as hit when entry <= exit widened by a few ulps, so that
+// rounding cannot cull a true hit.  PK = false computes the same values with box_test, one child at a
+// time (for the register-bound one-thread-per-path kernels' two-level walks, where the packed pairs cost
+// spills).
 __device__ __forceinline__ unsigned long long pk2(float a, float b) {
     unsigned long long r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -72,27 +73,28 @@ __device__ __forceinline__ unsigned long long pk2(float a, float b) {
 __device__ __forceinline__ void unpk2(unsigned long long v, float& a, float& b) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
-__device__ __forceinline__ unsigned long long slab2(float lo0, float lo1, float o, float id) {
+__device__ __forceinline__ void slab2(float p0, float p1, float o0, float o1, float i0, float i1, float& t0,
+                                      float& t1) {
     unsigned long long d, r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk2(lo0, lo1)), "l"(pk2(o, o)));
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(d), "l"(pk2(id, id)));
-    return r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk2(p0, p1)), "l"(pk2(o0, o1)));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(d), "l"(pk2(i0, i1)));
+    unpk2(r, t0, t1);
 }
 template <bool PK = true>
-__device__ __forceinline__ void box_test2(float4 nx, float4 ny, float4 nz, float3 o, float3 id, float tmax,
+__device__ __forceinline__ void box_test2(float4 n0, float4 n1, float4 n2, float3 o, float3 id, float tmax,
                                           float& t0, float& t1, bool& h0, bool& h1) {
     if constexpr (!PK) {
-        h0 = box_test(nx.x, nx.z, ny.x, ny.z, nz.x, nz.z, o, id, tmax, t0);
-        h1 = box_test(nx.y, nx.w, ny.y, ny.w, nz.y, nz.w, o, id, tmax, t1);
+        h0 = box_test(n0.x, n0.z, n0.y, n0.w, n2.x, n2.y, o, id, tmax, t0);
+        h1 = box_test(n1.x, n1.z, n1.y, n1.w, n2.z, n2.w, o, id, tmax, t1);
         return;
     }
     float xa0, xa1, xb0, xb1, ya0, ya1, yb0, yb1, za0, za1, zb0, zb1;
-    unpk2(slab2(nx.x, nx.y, o.x, id.x), xa0, xa1);
-    unpk2(slab2(nx.z, nx.w, o.x, id.x), xb0, xb1);
-    unpk2(slab2(ny.x, ny.y, o.y, id.y), ya0, ya1);
-    unpk2(slab2(ny.z, ny.w, o.y, id.y), yb0, yb1);
-    unpk2(slab2(nz.x, nz.y, o.z, id.z), za0, za1);
-    unpk2(slab2(nz.z, nz.w, o.z, id.z), zb0, zb1);
+    slab2(n0.x, n0.y, o.x, o.y, id.x, id.y, xa0, ya0);
+    slab2(n0.z, n0.w, o.x, o.y, id.x, id.y, xb0, yb0);
+    slab2(n1.x, n1.y, o.x, o.y, id.x, id.y, xa1, ya1);
+    slab2(n1.z, n1.w, o.x, o.y, id.x, id.y, xb1, yb1);
+    slab2(n2.x, n2.y, o.z, o.z, id.z, id.z, za0, zb0);
+    slab2(n2.z, n2.w, o.z, o.z, id.z, id.z, za1, zb1);
     const float a0 = fmaxf(fmaxf(fminf(xa0, xb0), fminf(ya0, yb0)), fmaxf(fminf(za0, zb0), 0.0f));
     const float e0 = fminf(fminf(fmaxf(xa0, xb0), fmaxf(ya0, yb0)), fminf(fmaxf(za0, zb0), tmax));
     const float a1 = fmaxf(fmaxf(fminf(xa1, xb1), fminf(ya1, yb1)), fmaxf(fminf(za1, zb1), 0.0f));
@@ -124,14 +126,17 @@ __device__ __forceinline__ bool tri_test(const float4* __restrict__ tris, uint32
     return true;
 }
 
+// One node: two 256-bit loads (node records are 64-byte aligned).
 __device__ __forceinline__ void load_node(const float4* __restrict__ nodes, uint32_t i, float4& n0, float4& n1,
                                           float4& n2, uint2& refs) {
     const float4* p = nodes + 4 * (size_t)i;
-    n0 = __ldg(p);
-    n1 = __ldg(p + 1);
-    n2 = __ldg(p + 2);
-    float4 n3 = __ldg(p + 3);
-    refs = make_uint2(__float_as_uint(n3.x), __float_as_uint(n3.y));
+    float pad0, pad1;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(n0.x), "=f"(n0.y), "=f"(n0.z), "=f"(n0.w), "=f"(n1.x), "=f"(n1.y), "=f"(n1.z), "=f"(n1.w)
+        : "l"(p));
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(n2.x), "=f"(n2.y), "=f"(n2.z), "=f"(n2.w), "=r"(refs.x), "=r"(refs.y), "=f"(pad0), "=f"(pad1)
+        : "l"(p + 2));
 }
 
 // ------------------------------------------------------------------ traversal stacks

@@ -1,0 +1,60 @@
+"""Pooled walks of the wavefront's dense trace launches (pt_pool.cuh): a warp hands queue slots to its lanes
+one by one, so slots at the ends of chunks, chunks at the ends of the queues and launches with fewer or more
+chunks than warps are where it could go wrong.  The megakernel walks one ray per thread and takes no slot from
+a pool; both compute the same FP32 operations, so radiance, signatures and ray counts must be equal bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2605_27323_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+# paths per launch: one, a chunk of 32 and its neighbours, about one and about two chunks per warp of a full grid
+# (152 SMs x 5 blocks x 8 warps x 32 = 194560 slots), and a queue that is no multiple of anything
+SIZES = [(1, 1, 1), (31, 1, 1), (32, 1, 1), (33, 1, 1), (311, 313, 1), (441, 441, 1), (4865, 40, 1), (487, 799, 1),
+         (523, 397, 3)]
+
+
+@pytest.fixture(scope="module")
+def views():
+    import torch
+
+    import paper_2605_27323_gb300 as pt
+    assert torch.cuda.is_available()
+    soup = scenes.random_soup(n_tris=3000, seed=11, spread=1.0, size=0.25)
+    out = {}
+    for name, sc in (("soup", soup), ("spheres", scenes.spheres_scene(seed=5, n_spheres=40, level=2, ground_quads=32,
+                                                                      extent=15.0))):
+        out[name] = (pt.Scene.from_dict(sc), sc.get("camera") or scenes.camera((0.2, 0.4, 4.0), (0, 0, 0)))
+    return out
+
+
+@pytest.mark.parametrize("scene", ["soup", "spheres"])
+@pytest.mark.parametrize("width,height,spp", SIZES)
+def test_pooled_walks_equal_the_megakernel(views, scene, width, height, spp):
+    import torch
+    g, cam = views[scene]
+    cam = dict(cam, width=width, height=height)
+    a = g.render(cam, spp, 4, 3, path_L=True, sig=True, mode="wavefront")
+    sa = g.stats()
+    b = g.render(cam, spp, 4, 3, path_L=True, sig=True, mode="megakernel")
+    sb = g.stats()
+    assert sa["status"] == 0 and sb["status"] == 0
+    for k in ("img", "path_L", "sig"):
+        assert torch.equal(a[k], b[k]), k
+    assert (sa["extension_rays"], sa["shadow_rays"]) == (sb["extension_rays"], sb["shadow_rays"])
+
+
+@pytest.mark.parametrize("width,height", [(33, 1), (441, 441), (487, 799)])
+def test_pooled_replay_equals_the_separate_order(views, width, height):
+    """The adjoint replay's pooled shadow walks mark vertex records; the separate order marks them in lockstep.
+    Gradients are sums of float atomics: 1e-5 of the largest covers a reordering of 4e5 terms (sqrt(n) 2^-24)."""
+    import torch
+    g, cam = views["spheres"]
+    cam = dict(cam, width=width, height=height)
+    grad = torch.ones((height, width, 3), device="cuda") / (width * height)
+    ga, ge = g.backward(cam, 1, 4, 3, grad)
+    ha, he = g.backward(cam, 1, 4, 3, grad, separate_shadow=True)
+    for x, y in ((ga, ha), (ge, he)):
+        assert float((x - y).abs().max()) <= 1e-5 * max(float(y.abs().max()), 1e-30)
+    assert np.isfinite(float(ga.sum()))
