@@ -133,7 +133,7 @@ struct pt_scene {
     uint32_t n_mats = 0;
     float light_area = 0.f;
     float env[3] = {0.f, 0.f, 0.f};
-    DevBuf nodes, tris, mats, lights, cdf, status;
+    DevBuf nodes, tris, mats, lights, cdf;
     DevBuf tlas, inst;          // two-level scenes: top-level nodes and instance records
     bool instanced = false;
     // workspaces (grown on demand, kept until destroy)
@@ -178,17 +178,17 @@ struct pt_scene {
         s.env_g = env[1];
         s.env_b = env[2];
         s.n_mats = n_mats;
-        s.status = status.as<uint32_t>();
+        s.status = status();
         s.tlas = instanced ? tlas.as<const float4>() : nullptr;
         s.inst = instanced ? inst.as<const float4>() : nullptr;
         s.trav = trav();
         return s;
     }
-    uint32_t* counts() const { return counters.as<uint32_t>(); }
-    unsigned long long* hist() const { return reinterpret_cast<unsigned long long*>(counters.as<char>() + 256); }
+    unsigned long long* hist() const { return reinterpret_cast<unsigned long long*>(counters.as<char>() + pt::kHistOffset); }
     unsigned long long* rays() const { return hist() + 128; }
 
-    pt_status ensure_counters() { return counters.ensure(256 + 8 * pt::kHistWords); }
+    uint32_t* status() const { return counters.as<uint32_t>() + pt::kStatusWord; }
+    pt_status ensure_counters() { return counters.ensure(pt::kCounterBytes); }
     unsigned long long* trav() const { return hist() + 132; }   // 4 traversal counters
     unsigned long long* next_path() const { return hist() + 130; }
     unsigned long long* finish_claim() const { return hist() + 131; }
@@ -384,8 +384,7 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
     if (cap >= (1ull << 32)) cap = ((1ull << 32) - (1ull << 20)) / p0.spp * p0.spp;
     PT_TRY(sc->ensure_wf(cap));
     pt::WfBuffers w = sc->wfb;
-    w.counts = sc->counts();
-    w.hist = sc->hist();
+    pt::carve_counters(sc->counters.p, w);
     w.sig = sig;
     w.capacity = (uint32_t)cap;
     const pt::DevScene ds = sc->view();
@@ -412,7 +411,7 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
                 if (b == 0) {     // no shadow rays are pending before the first shading
                     pt::Launch le = launch_for(sc, pt::K_EXTEND, o.block_size, 256, st, n);
                     le.pdl = kStagePdl;
-                    PT_CUDA(pt::launch_extend(le, ds, w, in, p));
+                    PT_CUDA(pt::launch_extend(le, ds, w, in, b, p));
                 } else {
                     pt::Launch lt = launch_for(sc, sc->instanced ? pt::K_TRACE_INST : pt::K_TRACE, o.block_size, 256, st,
                                                2ull * n);
@@ -423,7 +422,7 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
                 bool sorted_f = n_keys > 0;
                 if (sorted_f) {
                     PT_TRY(sc->ev_begin(ST_SORT, st, ev));
-                    PT_CUDA(pt::launch_sort(simple_launch(sc, st, n), ds, w, in, sort_mode, n_keys, p));
+                    PT_CUDA(pt::launch_sort(simple_launch(sc, st, n), ds, w, in, b, sort_mode, n_keys, p));
                     PT_TRY(sc->ev_end(ev, st));
                 }
                 pt::Launch ls = launch_for(sc, pt::K_SHADE, o.block_size, 256, st, n);
@@ -431,18 +430,17 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
                 PT_TRY(sc->ev_begin(ST_SHADE, st, ev));
                 PT_CUDA(pt::launch_shade(ls, ds, p, w, in, b, sorted_f));
                 PT_TRY(sc->ev_end(ev, st));
-                PT_CUDA(pt::launch_prepare_fused(st, w, b, kStagePdl));
-                sc->launches += 3 + (sorted_f ? 3 : 0);
+                sc->launches += 2 + (sorted_f ? 3 : 0);
                 continue;
             }
             pt::Launch le = launch_for(sc, short_stack_kernel(sc, pt::K_EXTEND, p.short_stack), o.block_size, 256, st, n);
             PT_TRY(sc->ev_begin(ST_EXTEND, st, ev));
-            PT_CUDA(pt::launch_extend(le, ds, w, in, p));
+            PT_CUDA(pt::launch_extend(le, ds, w, in, b, p));
             PT_TRY(sc->ev_end(ev, st));
             bool sorted = n_keys > 0;
             if (sorted) {
                 PT_TRY(sc->ev_begin(ST_SORT, st, ev));
-                PT_CUDA(pt::launch_sort(simple_launch(sc, st, n), ds, w, in, sort_mode, n_keys, p));
+                PT_CUDA(pt::launch_sort(simple_launch(sc, st, n), ds, w, in, b, sort_mode, n_keys, p));
                 PT_TRY(sc->ev_end(ev, st));
             }
             pt::Launch ls = launch_for(sc, pt::K_SHADE, o.block_size, 256, st, n);
@@ -453,8 +451,7 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
             PT_TRY(sc->ev_begin(ST_SHADOW, st, ev));
             PT_CUDA(pt::launch_shadow(lw, ds, p, w, b));
             PT_TRY(sc->ev_end(ev, st));
-            PT_CUDA(pt::launch_prepare(st, w, b));
-            sc->launches += 4 + (sorted ? 3 : 0);
+            sc->launches += 3 + (sorted ? 3 : 0);
             if (o.hybrid_threshold && b + 1 < p.max_depth) {
                 // hybrid: finish the remaining bounces in one kernel if few paths are left
                 const uint32_t thr = (uint32_t)std::min<uint64_t>(o.hybrid_threshold, 0xFFFFFFFFull);
@@ -470,11 +467,11 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
         PT_TRY(sc->ev_begin(ST_REDUCE, st, ev));
         if (accum)
             PT_CUDA(pt::launch_accumulate(simple_launch(sc, st, n / p.spp), reinterpret_cast<const float*>(w.L), 4,
-                                          w0 / p.spp, n / p.spp, p.spp, accum, count, img));
+                                          w0 / p.spp, n / p.spp, p.spp, accum, count, img, &w));
         else {
             pt::Launch lr = simple_launch(sc, st, n / p.spp);
             lr.pdl = kStagePdl;
-            PT_CUDA(pt::launch_reduce(lr, reinterpret_cast<const float*>(w.L), 4, w0 / p.spp, n / p.spp, p.spp, img));
+            PT_CUDA(pt::launch_reduce(lr, reinterpret_cast<const float*>(w.L), 4, w0 / p.spp, n / p.spp, p.spp, img, &w));
         }
         if (path_L) PT_CUDA(pt::launch_copy_L(simple_launch(sc, st, n), w.L, n, path_L + 3 * w0));
         PT_TRY(sc->ev_end(ev, st));
@@ -590,7 +587,7 @@ pt_status batch_render(pt_scene* const* scenes, const pt_camera* cams, const uin
         PT_TRY(carve_wavefront(ctx->wf, cap, ctx->wfb));
         ctx->capacity = cap;
     }
-    PT_TRY(ctx->counters.ensure(256 + 8 * pt::kHistWords));
+    PT_TRY(ctx->counters.ensure(pt::kCounterBytes));
     // wave segments: runs of pixels of one scene inside each wave
     std::vector<pt::BatchSegment> segs;
     struct Wave {
@@ -660,8 +657,7 @@ pt_status batch_render(pt_scene* const* scenes, const pt_camera* cams, const uin
     const unsigned long long* px_dev = reinterpret_cast<const unsigned long long*>(tb + o_px);
     const pt::BatchSegment* seg_dev = reinterpret_cast<const pt::BatchSegment*>(tb + o_seg);
     pt::WfBuffers w = ctx->wfb;
-    w.counts = ctx->counters.as<uint32_t>();
-    w.hist = reinterpret_cast<unsigned long long*>(ctx->counters.as<char>() + 256);
+    pt::carve_counters(ctx->counters.p, w);
     w.sig = nullptr;
     w.capacity = (uint32_t)cap;
     PT_CUDA(cudaMemsetAsync(ctx->counters.p, 0, ctx->counters.bytes, st));
@@ -786,7 +782,6 @@ pt_status render_impl(pt_scene* sc, const pt_camera* cam, uint32_t spp, uint32_t
     sc->last_paths = n_paths;
     sc->launches = 0;
     PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
-    PT_CUDA(cudaMemsetAsync(sc->status.p, 0, 4, st));
     if (accum && sample_offset == 0) PT_CUDA(cudaMemsetAsync(accum, 0, n_pixels * 12, st));
     pt::RenderParams p;
     p.seed = seed;
@@ -996,7 +991,6 @@ pt_status pt_scene_create(const float* verts, uint32_t n_verts, const uint32_t* 
     if ((s = sc->mats.ensure(dm.size() * sizeof(pt::DevMat))) != PT_OK) return bail(s);
     if ((s = sc->lights.ensure(std::max<size_t>(lrec.size() * 4, 48))) != PT_OK) return bail(s);
     if ((s = sc->cdf.ensure(cdf.size() * 4)) != PT_OK) return bail(s);
-    if ((s = sc->status.ensure(256)) != PT_OK) return bail(s);
     if ((s = sc->ensure_counters()) != PT_OK) return bail(s);
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->nodes.p, bvh.nodes.data(), bvh.nodes.size() * 4, cudaMemcpyHostToDevice, st);
@@ -1005,7 +999,6 @@ pt_status pt_scene_create(const float* verts, uint32_t n_verts, const uint32_t* 
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->mats.p, dm.data(), dm.size() * sizeof(pt::DevMat), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !lrec.empty()) e = cudaMemcpyAsync(sc->lights.p, lrec.data(), lrec.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->cdf.p, cdf.data(), cdf.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sc->status.p, 0, 256, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -1261,7 +1254,6 @@ pt_status pt_scene_create_instanced(uint32_t n_meshes, const float* const* verts
     if ((s = sc->mats.ensure(dm.size() * sizeof(pt::DevMat))) != PT_OK) return bail(s);
     if ((s = sc->lights.ensure(std::max<size_t>(lrec.size() * 4, 48))) != PT_OK) return bail(s);
     if ((s = sc->cdf.ensure(cdf.size() * 4)) != PT_OK) return bail(s);
-    if ((s = sc->status.ensure(256)) != PT_OK) return bail(s);
     if ((s = sc->ensure_counters()) != PT_OK) return bail(s);
     cudaError_t e = cudaMemcpyAsync(sc->nodes.p, nodes.data(), nodes.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->tris.p, trec.data(), trec.size() * 4, cudaMemcpyHostToDevice, st);
@@ -1270,7 +1262,6 @@ pt_status pt_scene_create_instanced(uint32_t n_meshes, const float* const* verts
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->mats.p, dm.data(), dm.size() * sizeof(pt::DevMat), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !lrec.empty()) e = cudaMemcpyAsync(sc->lights.p, lrec.data(), lrec.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->cdf.p, cdf.data(), cdf.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sc->status.p, 0, 256, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -1360,7 +1351,6 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
     sc->last_paths = n_paths;
     sc->launches = 0;
     PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
-    PT_CUDA(cudaMemsetAsync(sc->status.p, 0, 4, st));
     if (max_depth == 0 || sc->n_mats == 0) return PT_OK;
     pt::RenderParams p;
     p.seed = seed;
@@ -1389,8 +1379,7 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
         const size_t rec_bytes = align256(cap * max_depth * 64);
         PT_TRY(sc->adj.ensure(rec_bytes + align256(cap * 4)));
         pt::WfBuffers w = sc->wfb;
-        w.counts = sc->counts();
-        w.hist = sc->hist();
+        pt::carve_counters(sc->counters.p, w);
         w.sig = nullptr;
         w.capacity = (uint32_t)cap;
         pt::AdjBuffers ab;
@@ -1419,7 +1408,7 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
                 } else {
                     pt::Launch le = launch_for(sc, pt::K_EXTEND, o.block_size, 256, st, n);
                     le.pdl = fused && kStagePdl;
-                    PT_CUDA(pt::launch_extend(le, ds, w, in, pw));
+                    PT_CUDA(pt::launch_extend(le, ds, w, in, b, pw));
                 }
                 PT_TRY(sc->ev_end(e2, st));
                 PT_TRY(sc->ev_begin(ST_SHADE, st, e2));
@@ -1427,21 +1416,17 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
                 ls.pdl = fused && kStagePdl;
                 PT_CUDA(pt::launch_shade_adj(ls, ds, pw, w, ab, in, b));
                 PT_TRY(sc->ev_end(e2, st));
-                if (fused) {
-                    PT_CUDA(pt::launch_prepare_fused(st, w, b, kStagePdl));
-                    continue;
-                }
+                if (fused) continue;
                 PT_TRY(sc->ev_begin(ST_SHADOW, st, e2));
                 PT_CUDA(pt::launch_shadow_adj(launch_for(sc, pt::K_SHADOW_ADJ, o.block_size, 256, st, n), ds, pw, w, ab, b));
                 PT_TRY(sc->ev_end(e2, st));
-                PT_CUDA(pt::launch_prepare(st, w, b));
             }
             PT_TRY(sc->ev_begin(ST_REDUCE, st, e2));
             pt::Launch lr = simple_launch(sc, st, n);
             lr.pdl = fused && kStagePdl;
             PT_CUDA(pt::launch_adjoint_reverse(lr, ds, pw, w, ab, n, grad, d_grad_albedo, d_grad_emission));
             PT_TRY(sc->ev_end(e2, st));
-            sc->launches += 2 + (fused ? 3 : 4) * max_depth;
+            sc->launches += 2 + (fused ? 2 : 3) * max_depth;
         }
     }
     PT_TRY(sc->ev_end(ev, st));
@@ -1509,7 +1494,7 @@ pt_status pt_get_stats(pt_scene* sc, pt_stats* out) {
     std::vector<unsigned long long> h(pt::kHistWords);
     uint32_t status = 0;
     PT_CUDA(cudaMemcpy(h.data(), sc->hist(), pt::kHistWords * 8, cudaMemcpyDeviceToHost));
-    PT_CUDA(cudaMemcpy(&status, sc->status.p, 4, cudaMemcpyDeviceToHost));
+    PT_CUDA(cudaMemcpy(&status, sc->status(), 4, cudaMemcpyDeviceToHost));
     out->paths = sc->last_paths;
     out->launches_total = sc->launches;
     if (sc->last_mode != PT_MODE_WAVEFRONT) {

@@ -11,7 +11,7 @@ namespace pt {
 template <bool INST>
 __global__ void __launch_bounds__(256, 3) k_shade_adj(SingleSrc src, WfBuffers w, AdjBuffers a, int in, uint32_t b) {
     stage_prologue();
-    const uint32_t n = min(w.counts[0], w.capacity);
+    const uint32_t n = min(w.bc[b].active, w.capacity);
     const uint64_t base = src.base();
     const int out = in ^ 1;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(256, 3) k_shade_adj(SingleSrc src, WfBuffers w
                 if (!V.cont || V.last) a.pend[pid] = b + 1u;
             }
         }
-        const uint32_t k = warp_append(&w.counts[2], want_shadow);
+        uint32_t k, q;
+        warp_append2(&w.bc[b + 1], want_shadow, want_ray, k, q);
         if (want_shadow) {
             if (k < w.capacity) {
                 __stcs(&w.s_o[k], so);
@@ -74,7 +75,6 @@ __global__ void __launch_bounds__(256, 3) k_shade_adj(SingleSrc src, WfBuffers w
                 atomicOr(src.s.status, ST_QUEUE);
             }
         }
-        const uint32_t q = warp_append(&w.counts[1], want_ray);
         if (want_ray) {
             if (q < w.capacity) {
                 __stcs(&w.q_o[out][q], ro);
@@ -90,11 +90,11 @@ __global__ void __launch_bounds__(256, 3) k_shade_adj(SingleSrc src, WfBuffers w
 // Wavefront adjoint shadow stage: mark the vertex's NEE sample visible when unoccluded.
 template <bool INST>
 __global__ void __launch_bounds__(256) k_shadow_adj(SingleSrc src, WfBuffers w, AdjBuffers a, uint32_t b) {
-    const uint32_t n = min(w.counts[2], w.capacity);
+    const uint32_t n = min(w.bc[b + 1].shadow, w.capacity);
     if (n == 0u) return;
     const size_t cap = w.capacity;
     const uint32_t chunks = (n + 31u) / 32u;
-    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[5])) {
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim_shadow)) {
         const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         const float4 so = __ldcs(&w.s_o[j]), sd = __ldcs(&w.s_d[j]);

@@ -96,7 +96,7 @@ template <bool SIG, bool MIS, bool INST, int SK = 0>
 __global__ void __launch_bounds__(128, 8) k_finish(SingleSrc src, WfBuffers w, int in, uint32_t b0, uint32_t threshold,
                                                   unsigned long long* __restrict__ claim) {
     __shared__ unsigned int h_s[128];     // [b]: extension rays, [64 + b]: shadow rays of bounce b
-    const uint32_t n = min(w.counts[0], w.capacity);
+    const uint32_t n = min(w.bc[b0].active, w.capacity);
     if (n == 0u || n > threshold) return;  // the same value for every thread of the grid
     for (uint32_t k = threadIdx.x; k < 128u; k += blockDim.x) h_s[k] = 0u;
     __syncthreads();
@@ -160,9 +160,9 @@ __global__ void __launch_bounds__(128, 8) k_finish(SingleSrc src, WfBuffers w, i
         if (h_s[k]) atomicAdd(&w.hist[k], (unsigned long long)h_s[k]);
 }
 
-__global__ void k_finish_commit(WfBuffers w, uint32_t threshold, unsigned long long* claim) {
-    const uint32_t n = min(w.counts[0], w.capacity);
-    if (n > 0u && n <= threshold) w.counts[0] = 0u;
+__global__ void k_finish_commit(WfBuffers w, uint32_t b0, uint32_t threshold, unsigned long long* claim) {
+    const uint32_t n = min(w.bc[b0].active, w.capacity);
+    if (n > 0u && n <= threshold) w.bc[b0].active = 0u;
     *claim = 0ull;
 }
 
@@ -217,7 +217,7 @@ cudaError_t launch_finish(const Launch& l, const DevScene& s, const RenderParams
 #undef PT_FIN
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_finish_commit<<<1, 1, 0, l.st>>>(w, threshold, claim);
+    k_finish_commit<<<1, 1, 0, l.st>>>(w, b0, threshold, claim);
     return cudaGetLastError();
 }
 

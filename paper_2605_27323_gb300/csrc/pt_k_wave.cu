@@ -1,10 +1,11 @@
 // pt_k_wave.cu -- the wavefront pipeline (Sec. 2.3, 3, 3.1): raygen -> per bounce { extend ->
-// (key sort) -> shade -> shadow -> prepare } -> accumulate.  Stages are linked by structure-of-arrays
+// (key sort) -> shade -> shadow } -> accumulate.  Stages are linked by structure-of-arrays
 // queues of 16-byte records (128-bit coalesced loads and stores); compaction is a warp-aggregated
-// atomic append into the next queue (one atomic per warp instead of one per path), and the prepare
-// step rotates the two-slot active count without a host round trip.  Grids are persistent (a
-// multiple of the SM count) and stride over the device-side count, so no host read-back or
-// indirect launch is needed.  Also the batched variants (many scenes, one wavefront).
+// atomic append into the next queues (one atomic per warp instead of one per path and queue).  Every
+// bounce has counters of its own (BounceCounts), so nothing rotates them between two stages and there is
+// no host round trip.  Grids are persistent (a multiple of the SM count) and stride over the device-side
+// count, so no host read-back or indirect launch is needed.  Also the batched variants (many scenes, one
+// wavefront).
 #include <type_traits>
 
 #include "pt_common.cuh"
@@ -33,14 +34,10 @@ __global__ void __launch_bounds__(256) k_raygen(Src src, uint64_t base, uint32_t
         w.L[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (w.sig) w.sig[l.path] = 0u;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        w.counts[0] = n;
-        w.counts[1] = 0u;
-        w.counts[2] = 0u;
-        w.counts[4] = 0u;
-        w.counts[5] = 0u;
-        w.counts[6] = 0u;      // no shadow rays pending for the first trace launch
-        if (wave_base_dev) *wave_base_dev = base;
+    if (blockIdx.x == 0) {
+        for (uint32_t k = threadIdx.x; k < (uint32_t)kBounceSlots; k += blockDim.x)
+            w.bc[k] = BounceCounts{0u, k == 0u ? n : 0u, 0u, 0u};
+        if (threadIdx.x == 0 && wave_base_dev) *wave_base_dev = base;
     }
 }
 
@@ -129,9 +126,9 @@ constexpr int trace_blocks(bool inst, bool pooled) { return inst ? 4 : pooled ? 
 // SK > 0: the walks keep their top SK stack entries in dynamic shared memory (single-level only).
 // CNT: count the walks' node visits and triangle tests into the scene's traversal counters.
 template <class Src, bool INST, int SK = 0, bool CNT = false>
-__global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_extend(Src src, WfBuffers w, int in) {
+__global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_extend(Src src, WfBuffers w, int in, uint32_t b) {
     stage_prologue();
-    const uint32_t n = min(w.counts[0], w.capacity);
+    const uint32_t n = min(w.bc[b].active, w.capacity);
     if (n == 0u) return;       // an emptied queue: no claims (the same for every thread)
     const uint64_t base = src.base();
     const float4* __restrict__ qo = w.q_o[in];
@@ -139,12 +136,12 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_ex
     float2* __restrict__ hit = w.hit;
     const uint32_t chunks = (n + 31u) / 32u;
     if constexpr (!INST && SK == 0 && !CNT) {
-        ChunkPool q(&w.counts[4], chunks);
+        ChunkPool q(&w.bc[b].claim, chunks);
         pool_walk(src.scene(0), q, chunks, n, 0u, ExtendIo<Src>{src, qo, qd, hit, base});
         return;
     }
     typename std::conditional<CNT, TravCount, NoCount>::type cnt;
-    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[4])) {
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim)) {
         const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
@@ -158,11 +155,12 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_ex
 
 // Key sort before shading (counting sort): keys + block histograms, scan, scatter into `perm`.
 template <class Src, bool INST>
-__global__ void __launch_bounds__(256) k_sort_keys(Src src, WfBuffers w, int in, uint32_t mode, uint32_t n_keys) {
+__global__ void __launch_bounds__(256) k_sort_keys(Src src, WfBuffers w, int in, uint32_t b, uint32_t mode,
+                                                   uint32_t n_keys) {
     extern __shared__ uint32_t hist_s[];
     for (uint32_t k = threadIdx.x; k < n_keys; k += blockDim.x) hist_s[k] = 0u;
     __syncthreads();
-    const uint32_t n = min(w.counts[0], w.capacity);
+    const uint32_t n = min(w.bc[b].active, w.capacity);
     const uint64_t base = src.base();
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
@@ -212,8 +210,8 @@ __global__ void __launch_bounds__(1024) k_sort_scan(WfBuffers w, uint32_t n_keys
     }
 }
 
-__global__ void __launch_bounds__(256) k_sort_scatter(WfBuffers w) {
-    const uint32_t n = min(w.counts[0], w.capacity);
+__global__ void __launch_bounds__(256) k_sort_scatter(WfBuffers w, uint32_t b) {
+    const uint32_t n = min(w.bc[b].active, w.capacity);
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t base = warp * 32u; base < n; base += n_warps * 32u) {
@@ -319,11 +317,11 @@ __device__ __forceinline__ void put_ray(const Src& src, const WfBuffers& w, int 
 }
 
 // Shade: emission, NEE sample (-> shadow queue), BSDF sample, roulette, compaction of survivors: each
-// warp appends its survivors with one atomic per queue (warp-aggregated).
+// warp appends its survivors with one atomic for both queues (warp-aggregated).
 template <class Src, bool SIG, bool INST>
 __global__ void __launch_bounds__(256, 3) k_shade(Src src, WfBuffers w, int in, uint32_t b, bool sorted) {
     stage_prologue();
-    const uint32_t n = min(w.counts[0], w.capacity);
+    const uint32_t n = min(w.bc[b].active, w.capacity);
     const uint64_t base = src.base();
     const int out = in ^ 1;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -332,9 +330,9 @@ __global__ void __launch_bounds__(256, 3) k_shade(Src src, WfBuffers w, int in, 
         const uint32_t j = wb + lane_id();
         ShadeOut r;
         if (j < n) r = shade_entry<Src, SIG, INST>(src, w, in, b, sorted, base, j);
-        const uint32_t k = warp_append(&w.counts[2], r.want_shadow);
+        uint32_t k, q;
+        warp_append2(&w.bc[b + 1], r.want_shadow, r.want_ray, k, q);
         if (r.want_shadow) put_shadow(src, w, k, r);
-        const uint32_t q = warp_append(&w.counts[1], r.want_ray);
         if (r.want_ray) put_ray(src, w, out, q, r);
     }
 }
@@ -343,12 +341,12 @@ __global__ void __launch_bounds__(256, 3) k_shade(Src src, WfBuffers w, int in, 
 // At most one shadow ray per path per bounce, so the read-modify-write of L needs no atomics.
 template <class Src, bool SIG, bool INST, int SK = 0, bool CNT = false>
 __global__ void __launch_bounds__(256) k_shadow(Src src, WfBuffers w, uint32_t b) {
-    const uint32_t n = min(w.counts[2], w.capacity);
+    const uint32_t n = min(w.bc[b + 1].shadow, w.capacity);
     if (n == 0u) return;
     const uint64_t base = src.base();
     typename std::conditional<CNT, TravCount, NoCount>::type cnt;
     const uint32_t chunks = (n + 31u) / 32u;
-    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.counts[5])) {
+    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim_shadow)) {
         const uint32_t j = c * 32u + lane_id();
         if (j >= n) continue;
         const float4 so = __ldcs(&w.s_o[j]), sd = __ldcs(&w.s_d[j]), sc = __ldcs(&w.s_c[j]);
@@ -384,7 +382,7 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
     // one chunk sequence over both sets: the extension rays' chunks, then the shadow rays'
     const uint32_t c_ext = (n_ext + per - 1u) / per, c_all = c_ext + (n_shd + per - 1u) / per;
     uint32_t c = first_chunk();
-    for (; c < c_ext; c = next_chunk(&w.counts[4])) {
+    for (; c < c_ext; c = next_chunk(&w.bc[b].claim)) {
         const uint32_t j = c * per + sub;
         const bool valid = j < n_ext;
         float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f), d4 = make_float4(0.f, 0.f, 1.f, 0.f);
@@ -401,7 +399,7 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
             ++led;
         }
     }
-    for (; c < c_all; c = next_chunk(&w.counts[4])) {
+    for (; c < c_all; c = next_chunk(&w.bc[b].claim)) {
         const uint32_t k = (c - c_ext) * per + sub;
         const bool valid = k < n_shd;
         float4 so = make_float4(0.f, 0.f, 0.f, 0.f), sd = make_float4(0.f, 0.f, 1.f, 0.f);
@@ -437,8 +435,8 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
 }
 
 // Trace (the extend stage of bounce b fused with the shadow stage of bounce b - 1): one launch walks
-// the BVH for the continuation rays of bounce b (closest hit, queue `in`, counts[0] entries) and for
-// the shadow rays that shading cast at bounce b - 1 (any hit, the shadow queue, counts[6] entries).
+// the BVH for the continuation rays of bounce b (closest hit, queue `in`, bc[b].active entries) and for
+// the shadow rays that shading cast at bounce b - 1 (any hit, the shadow queue, bc[b].shadow entries).
 // The two sets are independent -- a shadow ray only adds its contribution to its path's radiance, and
 // only the next shading reads that radiance -- so each path still adds its terms in the order
 // emission(b - 1), NEE(b - 1), emission(b), as in the megakernel.  Single-level launches walk both sets
@@ -451,7 +449,7 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
 template <class Src, bool SIG, bool INST, bool CNT = false, bool ADJ = false>
 __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src, WfBuffers w, AdjBuffers a, int in, uint32_t b) {
     stage_prologue();
-    const uint32_t n_ext = min(w.counts[0], w.capacity), n_shd = min(w.counts[6], w.capacity);
+    const uint32_t n_ext = min(w.bc[b].active, w.capacity), n_shd = min(w.bc[b].shadow, w.capacity);
     if (n_ext + n_shd == 0u) return;       // the same for every thread
     const uint64_t base = src.base();
     // Lanes per walk: 1 while the walks fill the grid; once they are few (the sparse late bounces),
@@ -470,7 +468,7 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
     }
     if constexpr (!INST && !CNT) {
         const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
-        ChunkPool q(&w.counts[4], c_all);
+        ChunkPool q(&w.bc[b].claim, c_all);
         pool_walk(src.scene(0), q, c_ext, n_ext, n_shd,
                   TraceIo<Src, SIG, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, base}, w, a, b});
         return;
@@ -482,7 +480,7 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
     {
         const float4* __restrict__ qo = w.q_o[in];
         const float4* __restrict__ qd = w.q_d[in];
-        for (; c < c_ext; c = next_chunk(&w.counts[4])) {
+        for (; c < c_ext; c = next_chunk(&w.bc[b].claim)) {
             const uint32_t j = c * 32u + lane_id();
             if (j >= n_ext) continue;
             const float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
@@ -492,7 +490,7 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
             if (INST) w.hit_inst[j] = h.inst;
         }
     }
-    for (; c < c_all; c = next_chunk(&w.counts[4])) {
+    for (; c < c_all; c = next_chunk(&w.bc[b].claim)) {
         const uint32_t k = (c - c_ext) * 32u + lane_id();
         if (k >= n_shd) continue;
         const float4 so = __ldcs(&w.s_o[k]), sd = __ldcs(&w.s_d[k]);
@@ -520,35 +518,20 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
     flush_count(src.scene(0), ca, 2);
 }
 
-// Prepare after shading in the fused pipeline: record this bounce's counts, promote the next count,
-// and hand the shadow rays shading just cast to the next trace launch (counts[2] -> counts[6]).
-__global__ void k_prepare_fused(WfBuffers w, uint32_t b) {
-    stage_prologue();
-    w.hist[b] += w.counts[0];
-    w.hist[64 + b] += w.counts[2];
-    w.counts[0] = w.counts[1];
-    w.counts[1] = 0u;
-    w.counts[6] = w.counts[2];
-    w.counts[2] = 0u;
-    w.counts[4] = 0u;
-    w.counts[5] = 0u;
-}
-
-// Prepare (Sec. 3.1): record this bounce's counts, promote the next count, reset the slots.
-__global__ void k_prepare(WfBuffers w, uint32_t b) {
-    w.hist[b] += w.counts[0];
-    w.hist[64 + b] += w.counts[2];
-    w.counts[0] = w.counts[1];
-    w.counts[1] = 0u;
-    w.counts[2] = 0u;
-    w.counts[4] = 0u;      // the extend and shadow stages' work counters
-    w.counts[5] = 0u;
-}
-
 // ================================================================== accumulation
+// The end of a wave adds its bounces' counts to the call's totals (block 0 of the accumulation).
+__device__ __forceinline__ void fold_counts(const BounceCounts* bc, unsigned long long* hist) {
+    if (bc == nullptr || blockIdx.x != 0) return;
+    for (uint32_t b = threadIdx.x; b < 64u; b += blockDim.x) {
+        hist[b] += bc[b].active;
+        hist[64u + b] += bc[b + 1u].shadow;
+    }
+}
 __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ L, uint32_t stride_f, uint64_t pixel_begin,
-                                                uint64_t n_pixels, uint32_t spp, float* __restrict__ img) {
+                                                uint64_t n_pixels, uint32_t spp, float* __restrict__ img,
+                                                const BounceCounts* bc, unsigned long long* hist) {
     stage_prologue();
+    fold_counts(bc, hist);
     const float inv = 1.0f / (float)spp;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t px = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; px < n_pixels; px += stride) {
@@ -572,7 +555,9 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ L, uin
 // at the image of one call with k1 + k2 + ... samples, bit for bit.
 __global__ void __launch_bounds__(256) k_accumulate(const float* __restrict__ L, uint32_t stride_f,
                                                     uint64_t pixel_begin, uint64_t n_pixels, uint32_t spp,
-                                                    float* __restrict__ sum, uint32_t count, float* __restrict__ img) {
+                                                    float* __restrict__ sum, uint32_t count, float* __restrict__ img,
+                                                    const BounceCounts* bc, unsigned long long* hist) {
+    fold_counts(bc, hist);
     const float inv = 1.0f / (float)count;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t px = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; px < n_pixels; px += stride) {
@@ -669,24 +654,25 @@ cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParam
     return cudaGetLastError();
 }
 
-cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, const RenderParams& p) {
+cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce,
+                          const RenderParams& p) {
     SingleSrc src{s, DevCamera{}, p};
-    if (s.tlas) return launch_k(l, 0, k_extend<SingleSrc, true>, src, w, in);
-    if (p.count_trav) return launch_k(l, 0, k_extend<SingleSrc, false, 0, true>, src, w, in);
+    if (s.tlas) return launch_k(l, 0, k_extend<SingleSrc, true>, src, w, in, bounce);
+    if (p.count_trav) return launch_k(l, 0, k_extend<SingleSrc, false, 0, true>, src, w, in, bounce);
     if (p.short_stack)
-        return launch_k(l, stack_smem_bytes(kShortStack, l.block), k_extend<SingleSrc, false, kShortStack>, src, w, in);
-    return launch_k(l, 0, k_extend<SingleSrc, false>, src, w, in);
+        return launch_k(l, stack_smem_bytes(kShortStack, l.block), k_extend<SingleSrc, false, kShortStack>, src, w, in, bounce);
+    return launch_k(l, 0, k_extend<SingleSrc, false>, src, w, in, bounce);
 }
 
-cudaError_t launch_sort(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t mode, uint32_t n_keys,
-                        const RenderParams& p) {
+cudaError_t launch_sort(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce, uint32_t mode,
+                        uint32_t n_keys, const RenderParams& p) {
     cudaError_t e = cudaMemsetAsync(w.bucket, 0, sizeof(uint32_t) * n_keys, l.st);
     if (e != cudaSuccess) return e;
     SingleSrc src{s, DevCamera{}, p};
-    if (s.tlas) k_sort_keys<SingleSrc, true><<<l.grid, l.block, sizeof(uint32_t) * n_keys, l.st>>>(src, w, in, mode, n_keys);
-    else k_sort_keys<SingleSrc, false><<<l.grid, l.block, sizeof(uint32_t) * n_keys, l.st>>>(src, w, in, mode, n_keys);
+    if (s.tlas) k_sort_keys<SingleSrc, true><<<l.grid, l.block, sizeof(uint32_t) * n_keys, l.st>>>(src, w, in, bounce, mode, n_keys);
+    else k_sort_keys<SingleSrc, false><<<l.grid, l.block, sizeof(uint32_t) * n_keys, l.st>>>(src, w, in, bounce, mode, n_keys);
     k_sort_scan<<<1, 1024, 0, l.st>>>(w, n_keys);
-    k_sort_scatter<<<l.grid, l.block, 0, l.st>>>(w);
+    k_sort_scatter<<<l.grid, l.block, 0, l.st>>>(w, bounce);
     return cudaGetLastError();
 }
 
@@ -744,21 +730,16 @@ cudaError_t launch_bounce_batch(const Launch& le, const Launch& ls, const Launch
     if (fused && b > 0)   // lw: the fused launch (this bounce's extension and the last bounce's shadow walks)
         e = launch_k(lt, 0, k_trace<TableSrc, false, false>, src, w, AdjBuffers{}, in, b);
     else
-        e = launch_k(le, 0, k_extend<TableSrc, false>, src, w, in);
+        e = launch_k(le, 0, k_extend<TableSrc, false>, src, w, in, b);
     if (e != cudaSuccess) return e;
     if (n_keys) {
         if ((e = cudaMemsetAsync(w.bucket, 0, sizeof(uint32_t) * n_keys, lk.st)) != cudaSuccess) return e;
-        k_sort_keys<TableSrc, false><<<lk.grid, lk.block, sizeof(uint32_t) * n_keys, lk.st>>>(src, w, in, sort_mode, n_keys);
+        k_sort_keys<TableSrc, false><<<lk.grid, lk.block, sizeof(uint32_t) * n_keys, lk.st>>>(src, w, in, b, sort_mode, n_keys);
         k_sort_scan<<<1, 1024, 0, lk.st>>>(w, n_keys);
-        k_sort_scatter<<<lk.grid, lk.block, 0, lk.st>>>(w);
+        k_sort_scatter<<<lk.grid, lk.block, 0, lk.st>>>(w, b);
     }
     if ((e = launch_k(lsh, 0, k_shade<TableSrc, false, false>, src, w, in, b, n_keys > 0)) != cudaSuccess) return e;
-    if (fused) {
-        return launch_prepare_fused(le.st, w, b, pdl);
-    } else {
-        k_shadow<TableSrc, false, false><<<lw.grid, lw.block, 0, lw.st>>>(src, w, b);
-        k_prepare<<<1, 1, 0, le.st>>>(w, b);
-    }
+    if (!fused) k_shadow<TableSrc, false, false><<<lw.grid, lw.block, 0, lw.st>>>(src, w, b);
     return cudaGetLastError();
 }
 
@@ -795,28 +776,16 @@ cudaError_t launch_trace_adj(const Launch& l, const DevScene& s, const RenderPar
     return launch_k(l, 0, k_trace<SingleSrc, false, false, false, true>, src, w, a, in, bounce);
 }
 
-cudaError_t launch_prepare_fused(cudaStream_t st, const WfBuffers& w, uint32_t bounce, bool pdl) {
-    Launch l;
-    l.grid = 1;
-    l.block = 1;
-    l.st = st;
-    l.pdl = pdl;
-    return launch_k(l, 0, k_prepare_fused, w, bounce);
-}
-
-cudaError_t launch_prepare(cudaStream_t st, const WfBuffers& w, uint32_t bounce) {
-    k_prepare<<<1, 1, 0, st>>>(w, bounce);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_reduce(const Launch& l, const float* L, uint32_t stride, uint64_t pixel_begin, uint64_t n_pixels,
-                          uint32_t spp, float* img) {
-    return launch_k(l, 0, k_reduce, L, stride, pixel_begin, n_pixels, spp, img);
+                          uint32_t spp, float* img, const WfBuffers* w) {
+    return launch_k(l, 0, k_reduce, L, stride, pixel_begin, n_pixels, spp, img,
+                    w ? (const BounceCounts*)w->bc : nullptr, w ? w->hist : nullptr);
 }
 
 cudaError_t launch_accumulate(const Launch& l, const float* L, uint32_t stride, uint64_t pixel_begin, uint64_t n_pixels,
-                              uint32_t spp, float* sum, uint32_t count, float* img) {
-    k_accumulate<<<l.grid, l.block, 0, l.st>>>(L, stride, pixel_begin, n_pixels, spp, sum, count, img);
+                              uint32_t spp, float* sum, uint32_t count, float* img, const WfBuffers* w) {
+    k_accumulate<<<l.grid, l.block, 0, l.st>>>(L, stride, pixel_begin, n_pixels, spp, sum, count, img,
+                                               w ? w->bc : nullptr, w ? w->hist : nullptr);
     return cudaGetLastError();
 }
 

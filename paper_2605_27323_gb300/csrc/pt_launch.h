@@ -33,25 +33,24 @@ cudaError_t launch_debug_paths(cudaStream_t st, const DevScene& s, const DevCame
 
 // Wavefront stages (Sec. 2.3, 3.1).  `in` selects the ping-pong queue read this bounce.
 cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParams& p, uint32_t n, const WfBuffers& w);
-cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, const RenderParams& p);
-cudaError_t launch_sort(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t mode, uint32_t n_keys,
-                        const RenderParams& p);
+cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce,
+                          const RenderParams& p);
+cudaError_t launch_sort(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce, uint32_t mode,
+                        uint32_t n_keys, const RenderParams& p);
 cudaError_t launch_shade(const Launch& l, const DevScene& s, const RenderParams& p, const WfBuffers& w, int in,
                          uint32_t bounce, bool sorted);
 cudaError_t launch_shadow(const Launch& l, const DevScene& s, const RenderParams& p, const WfBuffers& w,
                           uint32_t bounce);
-cudaError_t launch_prepare(cudaStream_t st, const WfBuffers& w, uint32_t bounce);
 // The fused pipeline: the extend stage of bounce b and the shadow stage of bounce b - 1 in one launch
-// (the shadow rays pending in counts[6]), and the prepare step that hands shading's new shadow rays on.
+// (the shadow rays pending in the bounce's counters).
 cudaError_t launch_trace(const Launch& l, const DevScene& s, const RenderParams& p, const WfBuffers& w, int in,
                          uint32_t bounce);
-cudaError_t launch_prepare_fused(cudaStream_t st, const WfBuffers& w, uint32_t bounce, bool pdl = false);
 // The adjoint replay's fused launch: its shadow walks mark the records of bounce - 1.
 cudaError_t launch_trace_adj(const Launch& l, const DevScene& s, const RenderParams& p, const WfBuffers& w,
                              const AdjBuffers& a, int in, uint32_t bounce);
 
 // Batched wavefront over device scene tables (TableSrc): raygen of one wave (publishes the wave
-// base), one bounce of extend/(sort)/shade/shadow/prepare (capturable: no host-varying arguments),
+// base), one bounce of extend/(sort)/shade/shadow (capturable: no host-varying arguments),
 // accumulation of a wave into the scenes' running sums, and the final sums -> means.
 cudaError_t launch_raygen_batch(const Launch& l, const BatchTables& t, const RenderParams& p, uint64_t base, uint32_t n,
                                 const WfBuffers& w);
@@ -66,13 +65,14 @@ cudaError_t launch_scale_batch(const Launch& l, const BatchTables& t, const unsi
 
 // Accumulation (Sec. 2.3): img[pixel] = (1/spp) * sum_s L[pixel * spp + s], samples in order.
 // L has `stride` floats per path (3 or 4), wave-local; pixels [pixel_begin, pixel_begin + n_pixels).
+// With `w` (a wavefront's wave) its bounce counts are added to the call's totals.
 cudaError_t launch_reduce(const Launch& l, const float* L, uint32_t stride, uint64_t pixel_begin, uint64_t n_pixels,
-                          uint32_t spp, float* img);
+                          uint32_t spp, float* img, const WfBuffers* w = nullptr);
 // Copy wave-local float4 radiance into the caller's N_p x 3 buffer at path offset `path_begin`.
 cudaError_t launch_copy_L(const Launch& l, const float4* L4, uint64_t n, float* out_L3);
 // sum[px] += the pixel's spp samples (in order); img[px] = sum[px] / count unless img is null
 cudaError_t launch_accumulate(const Launch& l, const float* L, uint32_t stride, uint64_t pixel_begin, uint64_t n_pixels,
-                              uint32_t spp, float* sum, uint32_t count, float* img);
+                              uint32_t spp, float* sum, uint32_t count, float* img, const WfBuffers* w = nullptr);
 // Hybrid: finish every active path of the wave in one kernel when at most `threshold` are active
 // entering bounce b0 (queue `in`), then empty the queue; `claim` is a zeroed device u64.
 cudaError_t launch_finish(const Launch& l, const DevScene& s, const RenderParams& p, const WfBuffers& w, int in,

@@ -31,9 +31,9 @@ bool static_is_device_ptr(const void* p);
 
 namespace {
 
-constexpr size_t kStaticScratchBytes = 384ull << 20;
-constexpr size_t kHeaderBytes = 256 + 8 * pt::kHistWords;  // counters (incl. this call's status word), totals
-constexpr uint32_t kStatusWord = 16;            // counts[16]: device status word of this call
+// 384 MiB less 1408 bytes of records (the wave capacity that pt.h states), after the call's counters
+constexpr size_t kHeaderBytes = (pt::kCounterBytes + 255) / 256 * 256;   // status word, totals, bounce counters
+constexpr size_t kStaticScratchBytes = (384ull << 20) - 1408 + kHeaderBytes;
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
@@ -102,7 +102,7 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
         char msg[200];
         std::snprintf(msg, sizeof msg, "spp %u needs %llu bytes per pixel; the static scratch holds %llu paths (%zu MiB)",
                       spp, (unsigned long long)spp * pt::kWfBytesPerPath, (unsigned long long)cap_max,
-                      kStaticScratchBytes >> 20);
+                      ((kStaticScratchBytes + (1u << 20) - 1) >> 20));
         return pt::static_set_error(PT_ERR_INVALID_ARG, msg);
     }
     unsigned char* base = nullptr;
@@ -114,15 +114,14 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
 
     // the array: counters and histories, then the wavefront records in the allocating layout
     pt::WfBuffers w{};
-    w.counts = reinterpret_cast<uint32_t*>(base);
-    w.hist = reinterpret_cast<unsigned long long*>(base + 256);
+    pt::carve_counters(base, w);
     const size_t used = kHeaderBytes + pt::carve_wavefront_at(reinterpret_cast<char*>(base) + kHeaderBytes, cap, w);
     if (used > kStaticScratchBytes) return pt::static_set_error(PT_ERR_UNSUPPORTED, "static scratch layout overflow");
     w.sig = o.d_path_sig;
     w.capacity = (uint32_t)cap;
     // faults of this call (traversal cap, queue overflow) go to a word of the array, not to the
     // scene's status word, so pt_get_stats keeps describing the scene's last pt_render call
-    ds.status = w.counts + kStatusWord;
+    ds.status = reinterpret_cast<uint32_t*>(base) + pt::kStatusWord;
 
     cudaError_t e = cudaMemsetAsync(base, 0, kHeaderBytes, st);   // counters, status word, histories
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
@@ -186,22 +185,17 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
         for (uint32_t b = 0; b < max_depth; ++b) {
             const int in = (int)(b & 1u);
             if (!fused || b == 0) {          // no shadow rays are pending before the first shading
-                if ((e = pt::launch_extend(le, ds, w, in, p)) != cudaSuccess) return cuda_fail(e, "extend");
+                if ((e = pt::launch_extend(le, ds, w, in, b, p)) != cudaSuccess) return cuda_fail(e, "extend");
             } else if ((e = pt::launch_trace(lt, ds, p, w, in, b)) != cudaSuccess) {
                 return cuda_fail(e, "trace");
             }
-            if (n_keys && (e = pt::launch_sort(plain(n), ds, w, in, sort_mode, n_keys, p)) != cudaSuccess)
+            if (n_keys && (e = pt::launch_sort(plain(n), ds, w, in, b, sort_mode, n_keys, p)) != cudaSuccess)
                 return cuda_fail(e, "sort");
             if ((e = pt::launch_shade(ls, ds, p, w, in, b, n_keys > 0)) != cudaSuccess) return cuda_fail(e, "shade");
-            if (fused) {
-                if ((e = pt::launch_prepare_fused(st, w, b, le.pdl)) != cudaSuccess) return cuda_fail(e, "prepare");
-                continue;
-            }
-            if ((e = pt::launch_shadow(lw, ds, p, w, b)) != cudaSuccess) return cuda_fail(e, "shadow");
-            if ((e = pt::launch_prepare(st, w, b)) != cudaSuccess) return cuda_fail(e, "prepare");
+            if (!fused && (e = pt::launch_shadow(lw, ds, p, w, b)) != cudaSuccess) return cuda_fail(e, "shadow");
         }
         if ((e = pt::launch_reduce(lr, reinterpret_cast<const float*>(w.L), 4, w0 / spp, n / spp, spp,
-                                   d_out_rgb)) != cudaSuccess)
+                                   d_out_rgb, &w)) != cudaSuccess)
             return cuda_fail(e, "reduce");
     }
     return PT_OK;

@@ -65,12 +65,20 @@ enum : uint32_t { MAT_LAMBERT = 0, MAT_GGX = 1, MAT_DIELECTRIC = 2 };
 constexpr uint32_t SAMPLER_HALTON_ID = 1;   // RenderParams::sampler value of the Halton jitter
 enum : uint32_t { ST_TRAVERSAL = 1u, ST_QUEUE = 2u, ST_TIMEOUT = 4u };
 
+// The counters of one bounce.  Entry b of the wave's array holds the shadow rays that shading queued at
+// bounce b - 1 and the paths active entering bounce b -- appended to by one 64-bit atomic -- and the next
+// unclaimed chunk of the bounce's trace launch and of its separate shadow stage.  The paper's two-slot active count
+// (Sec. 3.1: a prepare step promotes the next count and resets it) unrolled over the bounces, so that no
+// launch between two stages has to rotate it (2 to 3 us a bounce); raygen clears the array.
+struct alignas(16) BounceCounts {
+    uint32_t shadow, active, claim, claim_shadow;
+};
+constexpr int kBounceSlots = 66;       // bounces 0 .. max_depth <= 64, and one spare
+
 // Wavefront buffers of one wave (Sec. 2.3 / 3.1): ping-pong ray queues, hit records, sort
-// scratch, the shadow-ray queue, per-path radiance, and the counters.  counts[0] = active paths of
-// the current bounce, counts[1] = next bounce's count (filled by compaction), counts[2] = shadow
-// rays; the prepare step promotes [1] to [0] and resets [1] and [2] (the two-slot count of
-// Sec. 3.1).  The paper reuses one index buffer in place; here the two ray queues alternate, since
-// on CUDA a block may append into a slot that a block not yet scheduled still has to read.
+// scratch, the shadow-ray queue, per-path radiance, and the counters.  The paper reuses one index buffer
+// in place; here the two ray queues alternate, since on CUDA a block may append into a slot that a block
+// not yet scheduled still has to read.
 struct WfBuffers {
     float4* q_o[2];          // o.xyz | path index (wave-local) bits
     float4* q_d[2];          // d.xyz | flags (bit 0: previous vertex was delta)
@@ -84,8 +92,7 @@ struct WfBuffers {
     float4* s_d;             // shadow ray: d.xyz | path index bits
     float4* s_c;             // shadow ray: contribution.rgb | light index bits
     float4* L;               // per path (wave-local): radiance.rgb | -
-    uint32_t* counts;        // [0] active, [1] next, [2] shadow, [3] sort key count, [4] [5] work claims,
-                             // [6] shadow rays pending for the fused trace launch
+    BounceCounts* bc;        // kBounceSlots entries
     unsigned long long* hist;  // kHistWords per-call totals (layout at kHistWords)
     uint32_t* sig;           // per path (global id) branch signature, or null
     uint32_t capacity;
@@ -131,12 +138,23 @@ constexpr uint32_t kMaxEvents = 64;     // event-log capacity per path (testing 
 // Device bytes of one wave's records per path: two ping-pong ray queues of three float4 arrays, the
 // hit record (float2), the hit instance, sort key and permutation (u32 each), the shadow queue (three
 // float4 arrays) and the radiance (float4).
-// Per-call device totals (64-bit words after the 256-byte count block): [b] extension rays of bounce
+// The counter block of a call: 256 bytes of words (kStatusWord: the status word; byte 128: the batch's wave
+// base), the per-call totals, then the wave's BounceCounts.
+constexpr uint32_t kStatusWord = 16;
+// Per-call device totals (64-bit words after the 256-byte block): [b] extension rays of bounce
 // b, [64 + b] shadow rays of bounce b, [128] [129] megakernel ray totals, [130] next path to start,
 // [131] hybrid claim, [132, 136) traversal counters, [136, 141) walks the fused trace stage traced
 // with groups of 2, 4, 8, 16, 32 lanes per ray.
 constexpr int kHistWords = 144;
 constexpr int kHistGroupWalks = 136;
+constexpr size_t kHistOffset = 256;
+constexpr size_t kBounceOffset = kHistOffset + 8 * kHistWords;
+constexpr size_t kCounterBytes = kBounceOffset + kBounceSlots * sizeof(BounceCounts);
+static_assert(kBounceOffset % 16 == 0, "the bounce counters are 16-byte aligned");
+inline void carve_counters(void* base, WfBuffers& w) {
+    w.hist = reinterpret_cast<unsigned long long*>(static_cast<char*>(base) + kHistOffset);
+    w.bc = reinterpret_cast<BounceCounts*>(static_cast<char*>(base) + kBounceOffset);
+}
 
 constexpr size_t kWfBytesPerPath = 2 * 3 * 16 + 8 + 3 * 4 + 3 * 16 + 16;
 static_assert(kWfBytesPerPath == 180, "wavefront record layout changed: update the documented sizes");
