@@ -396,6 +396,9 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
         const uint32_t n = (uint32_t)std::min<uint64_t>(cap, n_paths - w0);
         pt::RenderParams p = p0;
         p.path_begin = w0;
+        p.ex = cam.ex;
+        p.ey = cam.ey;
+        p.ez = cam.ez;
         size_t ev = 0;
         PT_TRY(sc->ev_begin(ST_RAYGEN, st, ev));
         PT_CUDA(pt::launch_raygen(simple_launch(sc, st, n), cam, p, n, w));
@@ -1390,6 +1393,9 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
             const uint32_t n = (uint32_t)std::min<uint64_t>(cap, n_paths - w0);
             pt::RenderParams pw = p;
             pw.path_begin = w0;
+            pw.ex = dc.ex;
+            pw.ey = dc.ey;
+            pw.ez = dc.ez;
             size_t e2 = 0;
             PT_TRY(sc->ev_begin(ST_RAYGEN, st, e2));
             PT_CUDA(pt::launch_raygen(simple_launch(sc, st, n), dc, pw, n, w));

@@ -272,7 +272,8 @@ struct SingleSrc {
     __device__ __forceinline__ RenderParams params(uint32_t) const { return p; }
     // scene id carried in the queue records: none needed for one scene
     __device__ __forceinline__ uint32_t ray_tag(uint32_t, uint32_t flags) const { return flags; }
-    __device__ __forceinline__ uint32_t sid_from_ray(float, uint64_t, uint32_t) const { return 0; }
+    __device__ __forceinline__ uint32_t sid_from_ray(float) const { return 0; }
+    __device__ __forceinline__ float3 eye(uint32_t) const { return f3(p.ex, p.ey, p.ez); }
     __device__ __forceinline__ uint32_t shadow_tag(uint32_t light_j, uint32_t) const { return light_j; }
     __device__ __forceinline__ uint32_t sid_from_shadow(float, uint64_t, uint32_t) const { return 0; }
     __device__ __forceinline__ PathLoc locate_in(uint64_t base, uint32_t pid, uint32_t) const { return locate(base, pid); }
@@ -312,8 +313,9 @@ struct TableSrc {
     }
     // the scene id rides in the records' spare bits: ray d.w = flags | sid << 8; shadow c.w = sid
     __device__ __forceinline__ uint32_t ray_tag(uint32_t sid, uint32_t flags) const { return flags | (sid << 8); }
-    __device__ __forceinline__ uint32_t sid_from_ray(float dw, uint64_t, uint32_t) const {
-        return __float_as_uint(dw) >> 8;
+    __device__ __forceinline__ uint32_t sid_from_ray(float dw) const { return __float_as_uint(dw) >> 8; }
+    __device__ __forceinline__ float3 eye(uint32_t sid) const {
+        return f3(t.cams[sid].ex, t.cams[sid].ey, t.cams[sid].ez);
     }
     __device__ __forceinline__ uint32_t shadow_tag(uint32_t, uint32_t sid) const { return sid; }
     __device__ __forceinline__ uint32_t sid_from_shadow(float cw, uint64_t, uint32_t) const {

@@ -22,7 +22,15 @@ __global__ void __launch_bounds__(256, 3) k_shade_adj(SingleSrc src, WfBuffers w
         bool want_ray = false, want_shadow = false;
         float4 ro, rd, rtp, so, sd;
         if (j < n) {
-            const float4 o4 = __ldcs(&w.q_o[in][j]), d4 = __ldcs(&w.q_d[in][j]), tp4 = __ldcs(&w.q_tp[in][j]);
+            const float4 d4 = __ldcs(&w.q_d[in][j]);
+            float4 o4, tp4;
+            if (b == 0u) {       // a camera ray (see k_raygen)
+                o4 = f4(src.eye(0u), __uint_as_float(j));
+                tp4 = make_float4(1.f, 1.f, 1.f, 0.f);
+            } else {
+                o4 = __ldcs(&w.q_o[in][j]);
+                tp4 = __ldcs(&w.q_tp[in][j]);
+            }
             const float2 hh = __ldcs(&w.hit[j]);
             const uint32_t pid = __float_as_uint(o4.w);
             const uint32_t tri = __float_as_uint(hh.y);

@@ -176,6 +176,9 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
     for (uint64_t w0 = 0; w0 < n_paths; w0 += cap) {
         const uint32_t n = (uint32_t)std::min<uint64_t>(cap, n_paths - w0);
         p.path_begin = w0;
+        p.ex = dc.ex;
+        p.ey = dc.ey;
+        p.ez = dc.ez;
         pt::Launch le = persistent(per_extend, n), ls = persistent(per_shade, n);
         const pt::Launch lw = persistent(per_shadow, n);
         pt::Launch lt = persistent(per_trace, 2ull * n), lr = plain(n / spp);

@@ -58,6 +58,7 @@ struct RenderParams {
     uint32_t sampler = 0;         // pixel jitter: 0 PCG uniforms, 1 Halton (2,3) + Cranley-Patterson
     uint32_t mis = 0;             // 1: NEE and BSDF-sampled light hits combined by the power heuristic
     uint32_t short_stack = 0;     // 1: single-level walks keep their top stack entries in shared memory
+    float ex = 0.f, ey = 0.f, ez = 0.f;   // the camera's eye: the origin of every ray of bounce 0
     uint32_t count_trav = 0;      // 1: single-level walks count visited nodes and tested triangles
 };
 
@@ -80,9 +81,10 @@ constexpr int kBounceSlots = 66;       // bounces 0 .. max_depth <= 64, and one 
 // in place; here the two ray queues alternate, since on CUDA a block may append into a slot that a block
 // not yet scheduled still has to read.
 struct WfBuffers {
-    float4* q_o[2];          // o.xyz | path index (wave-local) bits
+    float4* q_o[2];          // o.xyz | path index (wave-local) bits (bounce 0: not stored, the eye and the slot)
     float4* q_d[2];          // d.xyz | flags (bit 0: previous vertex was delta)
-    float4* q_tp[2];         // throughput.xyz | solid-angle density of the BSDF sample (MIS weights)
+    float4* q_tp[2];         // throughput.xyz | solid-angle density of the BSDF sample (MIS weights); bounce 0:
+                             // not stored, (1, 1, 1 | 0)
     float2* hit;             // per queue slot: t, reordered triangle bits (0xFFFFFFFF: miss)
     uint32_t* hit_inst;      // per queue slot: instance of the hit (two-level scenes only)
     uint32_t* keys;          // per queue slot: sort key
