@@ -42,12 +42,13 @@ __global__ void __launch_bounds__(256) k_raygen(Src src, uint64_t base, uint32_t
 }
 
 // Extension rays as the pooled walks take them: a queue slot's ray (and its scene's tree), its hit record.
-template <class Src>
+template <class Src, bool INST>
 struct ExtendIo {
     const Src& src;
     const float4* __restrict__ qo;      // null at bounce 0: camera rays
     const float4* __restrict__ qd;
     float2* __restrict__ hit;
+    uint32_t* __restrict__ hit_inst;
     uint64_t base;
     __device__ __forceinline__ void fetch(uint32_t j, float3& o, float3& d, float& tbest, uint32_t& best,
                                           const float4*& nodes, const float4*& tris) const {
@@ -63,15 +64,16 @@ struct ExtendIo {
             tris = s.tris;
         }
     }
-    __device__ __forceinline__ void emit(uint32_t j, float t, uint32_t tri) const {
+    __device__ __forceinline__ void emit(uint32_t j, float t, uint32_t tri, uint32_t inst) const {
         hit[j] = make_float2(t, __uint_as_float(tri));
+        if (INST) hit_inst[j] = inst;
     }
 };
 
 // Extension rays and shadow rays (slots with kAnySlot; `best` carries their path, tbest < 0: occluded).
-template <class Src, bool SIG, bool ADJ>
+template <class Src, bool SIG, bool INST, bool ADJ>
 struct TraceIo {
-    ExtendIo<Src> ext;
+    ExtendIo<Src, INST> ext;
     const WfBuffers& w;
     const AdjBuffers& a;
     uint32_t b;
@@ -93,9 +95,9 @@ struct TraceIo {
             tris = s.tris;
         }
     }
-    __device__ __forceinline__ void emit(uint32_t slot, float t, uint32_t tri) const {
+    __device__ __forceinline__ void emit(uint32_t slot, float t, uint32_t tri, uint32_t inst) const {
         if (!(slot & kAnySlot)) {
-            ext.emit(slot, t, tri);
+            ext.emit(slot, t, tri, inst);
             return;
         }
         const bool occ = t < 0.0f;
@@ -136,23 +138,22 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_ex
     const float4* __restrict__ qd = w.q_d[in];
     float2* __restrict__ hit = w.hit;
     const uint32_t chunks = (n + 31u) / 32u;
-    if constexpr (!INST && SK == 0 && !CNT) {
+    if constexpr (SK == 0 && !CNT) {
         ChunkPool q(&w.bc[b].claim, chunks);
-        pool_walk(src.scene(0), q, chunks, n, 0u, ExtendIo<Src>{src, qo, qd, hit, base});
-        return;
+        pool_walk<INST>(src.scene(0), q, chunks, n, 0u, ExtendIo<Src, INST>{src, qo, qd, hit, w.hit_inst, base});
+    } else {       // single-level, in lockstep
+        typename std::conditional<CNT, TravCount, NoCount>::type cnt;
+        for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim)) {
+            const uint32_t j = c * 32u + lane_id();
+            if (j >= n) continue;
+            const float4 d4 = __ldcs(&qd[j]);
+            const uint32_t sid = src.sid_from_ray(d4.w);
+            const float3 o = qo ? xyz(__ldcs(&qo[j])) : src.eye(sid);
+            const Hit h = trace_closest<false, SK>(src.scene(sid), o, xyz(d4), cnt);
+            hit[j] = make_float2(h.t, __uint_as_float(h.tri));
+        }
+        flush_count(src.scene(0), cnt, 0);
     }
-    typename std::conditional<CNT, TravCount, NoCount>::type cnt;
-    for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim)) {
-        const uint32_t j = c * 32u + lane_id();
-        if (j >= n) continue;
-        const float4 d4 = __ldcs(&qd[j]);
-        const uint32_t sid = src.sid_from_ray(d4.w);
-        const float3 o = qo ? xyz(__ldcs(&qo[j])) : src.eye(sid);
-        Hit h = trace_closest<INST, SK>(src.scene(sid), o, xyz(d4), cnt);
-        hit[j] = make_float2(h.t, __uint_as_float(h.tri));
-        if (INST) w.hit_inst[j] = h.inst;
-    }
-    flush_count(src.scene(0), cnt, 0);
 }
 
 // Key sort before shading (counting sort): keys + block histograms, scan, scatter into `perm`.
@@ -451,9 +452,9 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
 // the shadow rays that shading cast at bounce b - 1 (any hit, the shadow queue, bc[b].shadow entries).
 // The two sets are independent -- a shadow ray only adds its contribution to its path's radiance, and
 // only the next shading reads that radiance -- so each path still adds its terms in the order
-// emission(b - 1), NEE(b - 1), emission(b), as in the megakernel.  Single-level launches walk both sets
-// through one pool (pool_walk): the continuation rays first, then the shadow rays; two-level and counting
-// launches take 32 continuation rays at a time until none is left and then 32 shadow rays at a time.
+// emission(b - 1), NEE(b - 1), emission(b), as in the megakernel.  Launches walk both sets
+// through one pool (pool_walk): the continuation rays first, then the shadow rays; the counting launches
+// take 32 continuation rays at a time until none is left and then 32 shadow rays at a time.
 // A launch therefore ends when both sets are done, and the shadow walks fill the extension walks' tail
 // instead of running after a stage boundary.
 // ADJ: the adjoint replay's variant, whose shadow walks mark the vertex record's NEE sample visible
@@ -478,56 +479,32 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
         trace_groups<Src, SIG, INST, ADJ>(src, w, a, in, b, n_ext, n_shd, G);
         return;
     }
-    if constexpr (!INST && !CNT) {
-        const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
-        ChunkPool q(&w.bc[b].claim, c_all);
-        pool_walk(src.scene(0), q, c_ext, n_ext, n_shd,
-                  TraceIo<Src, SIG, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, base}, w, a, b});
-        return;
-    }
-    typename std::conditional<CNT, TravCount, NoCount>::type cc, ca;
-    // one chunk sequence over both sets: the extension rays' chunks, then the shadow rays'
     const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
-    uint32_t c = first_chunk();
-    {
-        const float4* __restrict__ qo = w.q_o[in];
-        const float4* __restrict__ qd = w.q_d[in];
+    if constexpr (!CNT) {
+        ChunkPool q(&w.bc[b].claim, c_all);
+        pool_walk<INST>(src.scene(0), q, c_ext, n_ext, n_shd,
+                        TraceIo<Src, SIG, INST, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, w.hit_inst, base}, w, a, b});
+    } else {       // counting (single-level, no signatures), in lockstep
+        TravCount cc, ca;
+        uint32_t c = first_chunk();
         for (; c < c_ext; c = next_chunk(&w.bc[b].claim)) {
             const uint32_t j = c * 32u + lane_id();
             if (j >= n_ext) continue;
-            const float4 o4 = __ldcs(&qo[j]), d4 = __ldcs(&qd[j]);
-            Hit h = trace_closest<INST, 0>(src.scene(src.sid_from_ray(d4.w)), xyz(o4),
-                                           xyz(d4), cc);
+            const float4 o4 = __ldcs(&w.q_o[in][j]), d4 = __ldcs(&w.q_d[in][j]);
+            const Hit h = trace_closest<false, 0>(src.scene(src.sid_from_ray(d4.w)), xyz(o4), xyz(d4), cc);
             w.hit[j] = make_float2(h.t, __uint_as_float(h.tri));
-            if (INST) w.hit_inst[j] = h.inst;
         }
-    }
-    for (; c < c_all; c = next_chunk(&w.bc[b].claim)) {
-        const uint32_t k = (c - c_ext) * 32u + lane_id();
-        if (k >= n_shd) continue;
-        const float4 so = __ldcs(&w.s_o[k]), sd = __ldcs(&w.s_d[k]);
-        const uint32_t pid = __float_as_uint(sd.w);
-        if constexpr (ADJ) {
-            if (!trace_any<INST, 0>(src.scene(0), xyz(so), xyz(sd), so.w, ca)) {
-                float* fl = reinterpret_cast<float*>(a.rec + 4 * ((size_t)(b - 1u) * w.capacity + pid) + 3) + 3;
-                *fl = __uint_as_float(__float_as_uint(*fl) | 2u);
-            }
-        } else {
-            const float4 sc = __ldcs(&w.s_c[k]);
-            const bool occ =
-                trace_any<INST, 0>(src.scene(src.sid_from_shadow(sc.w, base, pid)), xyz(so), xyz(sd), so.w, ca);
-            if (!occ) {
-                float3 L = add_rn(xyz(w.L[pid]), xyz(sc));
-                w.L[pid] = f4(L, 0.f);
-            }
-            if (SIG) {
-                const uint32_t lj = __float_as_uint(sc.w);
-                w.sig[base + pid] ^= sig_event(b - 1u, 1, (lj << 2) | 2u | (occ ? 0u : 1u));
-            }
+        for (; c < c_all; c = next_chunk(&w.bc[b].claim)) {
+            const uint32_t k = (c - c_ext) * 32u + lane_id();
+            if (k >= n_shd) continue;
+            const float4 so = __ldcs(&w.s_o[k]), sd = __ldcs(&w.s_d[k]), sc = __ldcs(&w.s_c[k]);
+            const uint32_t pid = __float_as_uint(sd.w);
+            if (!trace_any<false, 0>(src.scene(src.sid_from_shadow(sc.w, base, pid)), xyz(so), xyz(sd), so.w, ca))
+                w.L[pid] = f4(add_rn(xyz(w.L[pid]), xyz(sc)), 0.f);
         }
+        flush_count(src.scene(0), cc, 0);
+        flush_count(src.scene(0), ca, 2);
     }
-    flush_count(src.scene(0), cc, 0);
-    flush_count(src.scene(0), ca, 2);
 }
 
 // ================================================================== accumulation

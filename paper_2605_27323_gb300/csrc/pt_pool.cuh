@@ -64,23 +64,62 @@ __device__ __forceinline__ uint32_t pool_take(ChunkPool& q, uint32_t c_ext, uint
     return j;
 }
 
-template <class Io>
+// Original id of a hit, looked up only to decide ties: the triangle's, in a two-level scene offset by the
+// instance's first id.
+__device__ __forceinline__ uint32_t pool_prim(const DevScene& s, uint32_t inst, uint32_t prim) {
+    return __float_as_uint(__ldg(s.inst + 8 * (size_t)inst + 3).y) + prim;
+}
+template <bool INST>
+__device__ __forceinline__ uint32_t pool_id(const DevScene& s, const float4* tris, uint32_t best, uint32_t inst) {
+    if (best == kMiss) return kMiss;
+    const uint32_t prim = __float_as_uint(__ldg(tris + 3 * (size_t)best).w);
+    return INST ? pool_prim(s, inst, prim) : prim;
+}
+
+// INST: a two-level scene.  A lane at a top-level leaf takes its ray into the leaf's instance (in the leaf
+// phase) and walks the mesh's tree with the same stack, above the top-level entries (`floor` marks them);
+// when the mesh's part of the stack is empty it returns to the world ray, kept in wo / wd.  Visits and tests
+// are those of trace_closest_inst / trace_any_inst, in the same order.  Against those nested lockstep loops,
+// on the 1080p frame of 200 placed spheres: bounce 1 879 -> 556 us, the frame 2.29 -> 1.76 ms (1.90 ms at 5
+// blocks an SM with 144 bytes of spills).
+template <bool INST, class Io>
 __device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint32_t c_ext, uint32_t n_ext,
                                           uint32_t n_shd, const Io& io) {
-    uint2 stk[kStack];
-    int sp = 0;
+    uint2 stk[INST ? 2 * kStack : kStack];     // (reference, entry distance); each tree is shallower than kStack
+    int sp = 0, floor = 0;
     uint32_t ref = kDone, slot = kNoSlot, best = kMiss;
-    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o;
+    uint32_t cur = kMiss, binst = kMiss;       // INST: the instance the lane is in (kMiss: top level), the hit's
+    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o, wo = o, wd = o;
     float tbest = 0.f;
-    const float4 *nodes = s.nodes, *tris = s.tris;
+    const float4 *nodes = INST ? s.tlas : s.nodes, *tris = s.tris;
     uint32_t steps = 0;
-    auto pop = [&]() {
+    auto pop = [&]() {       // the next deferred subtree whose entry is not beyond the best hit
         ref = kDone;
-        while (sp > 0) {
-            const uint2 v = stk[--sp];
-            if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
-                ref = v.x;
-                break;
+        if constexpr (!INST) {
+            while (sp > 0) {
+                const uint2 v = stk[--sp];
+                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
+                    ref = v.x;
+                    return;
+                }
+            }
+        } else {
+            while (true) {
+                if (sp == floor) {
+                    if (cur == kMiss) return;
+                    cur = kMiss;               // the mesh is done: back to the top level
+                    floor = 0;
+                    nodes = s.tlas;
+                    o = wo;
+                    d = wd;
+                    id = ray_rcp(d);
+                    continue;
+                }
+                const uint2 v = stk[--sp];
+                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
+                    ref = v.x;
+                    return;
+                }
             }
         }
     };
@@ -89,7 +128,7 @@ __device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint3
         const bool all = idle == 0xFFFFFFFFu;
         if (all || ((uint32_t)__popc(idle) >= kIdleLanes && q.c < q.c_all)) {
             if (ref == kDone && slot != kNoSlot) {
-                io.emit(slot, tbest, best);
+                io.emit(slot, tbest, best, binst);
                 slot = kNoSlot;
             }
             if (q.c >= q.c_all) break;
@@ -100,6 +139,13 @@ __device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint3
                 id = ray_rcp(d);
                 ref = 0u;
                 sp = 0;
+                if (INST) {
+                    wo = o;
+                    wd = d;
+                    nodes = s.tlas;
+                    cur = binst = kMiss;
+                    floor = 0;
+                }
             }
             steps = 0;
         }
@@ -122,25 +168,39 @@ __device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint3
         } while ((uint32_t)__popc(m) >= kNodeLanes);
         if ((ref & kLeafBit) && ref != kDone) {
             const uint32_t first = (ref & 0x7FFFFFFFu) >> 3, n_leaf = (ref & 7u) + 1u;
-            const bool any = (slot & kAnySlot) != 0u;
-            bool over = false;
-            for (uint32_t k = 0; k < n_leaf && !over; ++k) {
-                float t;
-                uint32_t prim;
-                if (!tri_test(tris, first + k, o, d, t, prim) || !(t > 0.0f)) continue;
-                if (any) {
-                    over = t < tbest;
-                } else if (t < tbest ||
-                           (t == tbest && (best == kMiss || prim < __float_as_uint(__ldg(tris + 3 * (size_t)best).w)))) {
-                    tbest = t;
-                    best = first + k;
-                }
-            }
-            if (over) {
-                tbest = -1.0f;       // occluded
-                ref = kDone;
+            if (INST && cur == kMiss) {
+                // the leaf's instances one after the other (the builder makes leaves of one)
+                if (n_leaf > 1u) stk[sp++] = make_uint2(kLeafBit | (first + 1u) << 3 | (n_leaf - 2u), 0u);
+                const InstRay r = instance_ray(s, first, wo, wd);
+                cur = first;
+                floor = sp;
+                nodes = s.nodes;
+                o = r.o;
+                d = r.d;
+                id = ray_rcp(d);
+                ref = r.root;
             } else {
-                pop();
+                const bool any = (slot & kAnySlot) != 0u;
+                bool over = false;
+                for (uint32_t k = 0; k < n_leaf && !over; ++k) {
+                    float t;
+                    uint32_t prim;
+                    if (!tri_test(tris, first + k, o, d, t, prim) || !(t > 0.0f)) continue;
+                    if (any) {
+                        over = t < tbest;
+                    } else if (t < tbest || (t == tbest && pool_id<INST>(s, tris, best, binst) >
+                                                               (INST ? pool_prim(s, cur, prim) : prim))) {
+                        tbest = t;
+                        best = first + k;
+                        if (INST) binst = cur;
+                    }
+                }
+                if (over) {
+                    tbest = -1.0f;       // occluded
+                    ref = kDone;
+                } else {
+                    pop();
+                }
             }
         }
         if (++steps >= kMaxSteps) {

@@ -24,12 +24,14 @@ def views():
     soup = scenes.random_soup(n_tris=3000, seed=11, spread=1.0, size=0.25)
     out = {}
     for name, sc in (("soup", soup), ("spheres", scenes.spheres_scene(seed=5, n_spheres=40, level=2, ground_quads=32,
-                                                                      extent=15.0))):
+                                                                      extent=15.0)),
+                     ("placed", scenes.instanced_spheres_scene(seed=5, n_spheres=40, level=2, ground_quads=32,
+                                                               extent=15.0))):
         out[name] = (pt.Scene.from_dict(sc), sc.get("camera") or scenes.camera((0.2, 0.4, 4.0), (0, 0, 0)))
     return out
 
 
-@pytest.mark.parametrize("scene", ["soup", "spheres"])
+@pytest.mark.parametrize("scene", ["soup", "spheres", "placed"])
 @pytest.mark.parametrize("width,height,spp", SIZES)
 def test_pooled_walks_equal_the_megakernel(views, scene, width, height, spp):
     import torch
