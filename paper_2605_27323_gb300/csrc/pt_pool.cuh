@@ -30,6 +30,147 @@ constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 constexpr uint32_t kNodeLanes = 12;
 constexpr uint32_t kIdleLanes = 12;
 
+// Original id of a hit, looked up only to decide ties: the triangle's, in a two-level scene offset by the
+// instance's first id.
+__device__ __forceinline__ uint32_t pool_prim(const DevScene& s, uint32_t inst, uint32_t prim) {
+    return __float_as_uint(__ldg(s.inst + 8 * (size_t)inst + 3).y) + prim;
+}
+template <bool INST>
+__device__ __forceinline__ uint32_t pool_id(const DevScene& s, const float4* tris, uint32_t best, uint32_t inst) {
+    if (best == kMiss) return kMiss;
+    const uint32_t prim = __float_as_uint(__ldg(tris + 3 * (size_t)best).w);
+    return INST ? pool_prim(s, inst, prim) : prim;
+}
+
+// One lane's walk, stepped in the phases above by all 32 lanes together.  A closest-hit walk starts with
+// tbest = infinity and ends with the hit in (tbest, best, binst); an any-hit walk starts with its end distance in
+// tbest, which turns negative when an occluder is found (`best` is the caller's).
+// INST: a two-level scene.  A lane at a top-level leaf takes its ray into the leaf's instance (in the leaf
+// phase) and walks the mesh's tree with the same stack, above the top-level entries (`floor` marks them);
+// when the mesh's part of the stack is empty it returns to the world ray, kept in wo / wd.  Visits and tests
+// are those of trace_closest_inst / trace_any_inst, in the same order.  Against those nested lockstep loops,
+// on the 1080p frame of 200 placed spheres: bounce 1 879 -> 556 us, the frame 2.29 -> 1.76 ms (1.90 ms at 5
+// blocks an SM with 144 bytes of spills).
+template <bool INST>
+struct Walker {
+    // (reference, entry distance); each tree is shallower than kStack.  An array of its own beside the
+    // walker, whose other members then stay in registers.
+    using Stack = uint2[INST ? 2 * kStack : kStack];
+    int sp = 0, floor = 0;
+    uint32_t ref = kDone, best = kMiss;
+    uint32_t cur = kMiss, binst = kMiss;       // INST: the instance the lane is in (kMiss: top level), the hit's
+    float3 o, d, id, wo, wd;
+    float tbest = 0.f;
+    const float4 *nodes, *tris;
+
+    __device__ __forceinline__ explicit Walker(const DevScene& s)
+        : nodes(INST ? s.tlas : s.nodes), tris(s.tris) {
+        o = d = id = wo = wd = f3(0.f, 0.f, 0.f);
+    }
+    // Begin at the root; the caller has set o, d, tbest and best.
+    __device__ __forceinline__ void begin(const DevScene& s) {
+        id = ray_rcp(d);
+        ref = 0u;
+        sp = 0;
+        if (INST) {
+            wo = o;
+            wd = d;
+            nodes = s.tlas;
+            cur = binst = kMiss;
+            floor = 0;
+        }
+    }
+    // The next deferred subtree whose entry is not beyond the best hit.
+    __device__ __forceinline__ void pop(const DevScene& s, Stack& stk) {
+        ref = kDone;
+        if constexpr (!INST) {
+            while (sp > 0) {
+                const uint2 v = stk[--sp];
+                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
+                    ref = v.x;
+                    return;
+                }
+            }
+        } else {
+            while (true) {
+                if (sp == floor) {
+                    if (cur == kMiss) return;
+                    cur = kMiss;               // the mesh is done: back to the top level
+                    floor = 0;
+                    nodes = s.tlas;
+                    o = wo;
+                    d = wd;
+                    id = ray_rcp(d);
+                    continue;
+                }
+                const uint2 v = stk[--sp];
+                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
+                    ref = v.x;
+                    return;
+                }
+            }
+        }
+    }
+    // Node steps while at least kNodeLanes lanes hold an inner node.
+    __device__ __forceinline__ void node_phase(const DevScene& s, Stack& stk) {
+        uint32_t m;
+        do {
+            if (!(ref & kLeafBit)) {
+                float4 n0, n1, n2;
+                uint2 r;
+                load_node(nodes, ref, n0, n1, n2, r);
+                float t0, t1;
+                bool h0, h1;
+                box_test2(n0, n1, n2, o, id, tbest, t0, t1, h0, h1);
+                // the child to walk next (the nearer one when both boxes are hit) and the one deferred
+                const bool first0 = h0 && (t0 <= t1 || !h1);
+                ref = first0 ? r.x : r.y;
+                if (h0 && h1) stk[sp++] = make_uint2(first0 ? r.y : r.x, __float_as_uint(first0 ? t1 : t0));
+                else if (!(h0 || h1)) pop(s, stk);
+            }
+            m = __ballot_sync(0xFFFFFFFFu, !(ref & kLeafBit));
+        } while ((uint32_t)__popc(m) >= kNodeLanes);
+    }
+    // One leaf step of the lanes that hold a leaf; `any`: the lane's walk is an any-hit one.
+    __device__ __forceinline__ void leaf_phase(const DevScene& s, Stack& stk, bool any) {
+        if (!(ref & kLeafBit) || ref == kDone) return;
+        const uint32_t first = (ref & 0x7FFFFFFFu) >> 3, n_leaf = (ref & 7u) + 1u;
+        if (INST && cur == kMiss) {
+            // the leaf's instances one after the other (the builder makes leaves of one)
+            if (n_leaf > 1u) stk[sp++] = make_uint2(kLeafBit | (first + 1u) << 3 | (n_leaf - 2u), 0u);
+            const InstRay r = instance_ray(s, first, wo, wd);
+            cur = first;
+            floor = sp;
+            nodes = s.nodes;
+            o = r.o;
+            d = r.d;
+            id = ray_rcp(d);
+            ref = r.root;
+            return;
+        }
+        bool over = false;
+        for (uint32_t k = 0; k < n_leaf && !over; ++k) {
+            float t;
+            uint32_t prim;
+            if (!tri_test(tris, first + k, o, d, t, prim) || !(t > 0.0f)) continue;
+            if (any) {
+                over = t < tbest;
+            } else if (t < tbest || (t == tbest && pool_id<INST>(s, tris, best, binst) >
+                                                       (INST ? pool_prim(s, cur, prim) : prim))) {
+                tbest = t;
+                best = first + k;
+                if (INST) binst = cur;
+            }
+        }
+        if (over) {
+            tbest = -1.0f;       // occluded
+            ref = kDone;
+        } else {
+            pop(s, stk);
+        }
+    }
+};
+
 // A slot of the pool: an extension ray's queue index, or a shadow ray's with kAnySlot set (capacities stay
 // far below 2^31: a path's records take 180 bytes).
 constexpr uint32_t kAnySlot = 0x80000000u;
@@ -64,148 +205,34 @@ __device__ __forceinline__ uint32_t pool_take(ChunkPool& q, uint32_t c_ext, uint
     return j;
 }
 
-// Original id of a hit, looked up only to decide ties: the triangle's, in a two-level scene offset by the
-// instance's first id.
-__device__ __forceinline__ uint32_t pool_prim(const DevScene& s, uint32_t inst, uint32_t prim) {
-    return __float_as_uint(__ldg(s.inst + 8 * (size_t)inst + 3).y) + prim;
-}
-template <bool INST>
-__device__ __forceinline__ uint32_t pool_id(const DevScene& s, const float4* tris, uint32_t best, uint32_t inst) {
-    if (best == kMiss) return kMiss;
-    const uint32_t prim = __float_as_uint(__ldg(tris + 3 * (size_t)best).w);
-    return INST ? pool_prim(s, inst, prim) : prim;
-}
-
-// INST: a two-level scene.  A lane at a top-level leaf takes its ray into the leaf's instance (in the leaf
-// phase) and walks the mesh's tree with the same stack, above the top-level entries (`floor` marks them);
-// when the mesh's part of the stack is empty it returns to the world ray, kept in wo / wd.  Visits and tests
-// are those of trace_closest_inst / trace_any_inst, in the same order.  Against those nested lockstep loops,
-// on the 1080p frame of 200 placed spheres: bounce 1 879 -> 556 us, the frame 2.29 -> 1.76 ms (1.90 ms at 5
-// blocks an SM with 144 bytes of spills).
 template <bool INST, class Io>
 __device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint32_t c_ext, uint32_t n_ext,
                                           uint32_t n_shd, const Io& io) {
-    uint2 stk[INST ? 2 * kStack : kStack];     // (reference, entry distance); each tree is shallower than kStack
-    int sp = 0, floor = 0;
-    uint32_t ref = kDone, slot = kNoSlot, best = kMiss;
-    uint32_t cur = kMiss, binst = kMiss;       // INST: the instance the lane is in (kMiss: top level), the hit's
-    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o, wo = o, wd = o;
-    float tbest = 0.f;
-    const float4 *nodes = INST ? s.tlas : s.nodes, *tris = s.tris;
-    uint32_t steps = 0;
-    auto pop = [&]() {       // the next deferred subtree whose entry is not beyond the best hit
-        ref = kDone;
-        if constexpr (!INST) {
-            while (sp > 0) {
-                const uint2 v = stk[--sp];
-                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
-                    ref = v.x;
-                    return;
-                }
-            }
-        } else {
-            while (true) {
-                if (sp == floor) {
-                    if (cur == kMiss) return;
-                    cur = kMiss;               // the mesh is done: back to the top level
-                    floor = 0;
-                    nodes = s.tlas;
-                    o = wo;
-                    d = wd;
-                    id = ray_rcp(d);
-                    continue;
-                }
-                const uint2 v = stk[--sp];
-                if (__uint_as_float(v.y) <= tbest * 1.0000005f) {
-                    ref = v.x;
-                    return;
-                }
-            }
-        }
-    };
+    Walker<INST> k(s);
+    typename Walker<INST>::Stack stk;
+    uint32_t slot = kNoSlot, steps = 0;
     while (true) {
-        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, ref == kDone);
+        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, k.ref == kDone);
         const bool all = idle == 0xFFFFFFFFu;
         if (all || ((uint32_t)__popc(idle) >= kIdleLanes && q.c < q.c_all)) {
-            if (ref == kDone && slot != kNoSlot) {
-                io.emit(slot, tbest, best, binst);
+            if (k.ref == kDone && slot != kNoSlot) {
+                io.emit(slot, k.tbest, k.best, k.binst);
                 slot = kNoSlot;
             }
             if (q.c >= q.c_all) break;
             const uint32_t j = pool_take(q, c_ext, n_ext, n_shd, idle);
             if (j != kNoSlot) {
                 slot = j;
-                io.fetch(j, o, d, tbest, best, nodes, tris);
-                id = ray_rcp(d);
-                ref = 0u;
-                sp = 0;
-                if (INST) {
-                    wo = o;
-                    wd = d;
-                    nodes = s.tlas;
-                    cur = binst = kMiss;
-                    floor = 0;
-                }
+                io.fetch(j, k.o, k.d, k.tbest, k.best, k.nodes, k.tris);
+                k.begin(s);
             }
             steps = 0;
         }
-        uint32_t m;
-        do {
-            if (!(ref & kLeafBit)) {
-                float4 n0, n1, n2;
-                uint2 r;
-                load_node(nodes, ref, n0, n1, n2, r);
-                float t0, t1;
-                bool h0, h1;
-                box_test2(n0, n1, n2, o, id, tbest, t0, t1, h0, h1);
-                // the child to walk next (the nearer one when both boxes are hit) and the one deferred
-                const bool first0 = h0 && (t0 <= t1 || !h1);
-                ref = first0 ? r.x : r.y;
-                if (h0 && h1) stk[sp++] = make_uint2(first0 ? r.y : r.x, __float_as_uint(first0 ? t1 : t0));
-                else if (!(h0 || h1)) pop();
-            }
-            m = __ballot_sync(0xFFFFFFFFu, !(ref & kLeafBit));
-        } while ((uint32_t)__popc(m) >= kNodeLanes);
-        if ((ref & kLeafBit) && ref != kDone) {
-            const uint32_t first = (ref & 0x7FFFFFFFu) >> 3, n_leaf = (ref & 7u) + 1u;
-            if (INST && cur == kMiss) {
-                // the leaf's instances one after the other (the builder makes leaves of one)
-                if (n_leaf > 1u) stk[sp++] = make_uint2(kLeafBit | (first + 1u) << 3 | (n_leaf - 2u), 0u);
-                const InstRay r = instance_ray(s, first, wo, wd);
-                cur = first;
-                floor = sp;
-                nodes = s.nodes;
-                o = r.o;
-                d = r.d;
-                id = ray_rcp(d);
-                ref = r.root;
-            } else {
-                const bool any = (slot & kAnySlot) != 0u;
-                bool over = false;
-                for (uint32_t k = 0; k < n_leaf && !over; ++k) {
-                    float t;
-                    uint32_t prim;
-                    if (!tri_test(tris, first + k, o, d, t, prim) || !(t > 0.0f)) continue;
-                    if (any) {
-                        over = t < tbest;
-                    } else if (t < tbest || (t == tbest && pool_id<INST>(s, tris, best, binst) >
-                                                               (INST ? pool_prim(s, cur, prim) : prim))) {
-                        tbest = t;
-                        best = first + k;
-                        if (INST) binst = cur;
-                    }
-                }
-                if (over) {
-                    tbest = -1.0f;       // occluded
-                    ref = kDone;
-                } else {
-                    pop();
-                }
-            }
-        }
+        k.node_phase(s, stk);
+        k.leaf_phase(s, stk, (slot & kAnySlot) != 0u);
         if (++steps >= kMaxSteps) {
-            if (ref != kDone) atomicOr(s.status, ST_TRAVERSAL);
-            ref = kDone;
+            if (k.ref != kDone) atomicOr(s.status, ST_TRAVERSAL);
+            k.ref = kDone;
         }
     }
 }

@@ -1,7 +1,8 @@
 """Pooled walks of the wavefront's dense trace launches (pt_pool.cuh): a warp hands queue slots to its lanes
 one by one, so slots at the ends of chunks, chunks at the ends of the queues and launches with fewer or more
-chunks than warps are where it could go wrong.  The megakernel walks one ray per thread and takes no slot from
-a pool; both compute the same FP32 operations, so radiance, signatures and ray counts must be equal bit for bit."""
+chunks than warps are where it could go wrong.  The regenerating megakernel steps the walks of its lanes' paths in
+the same phases.  The megakernel in the paper's layout walks each ray to its end in one thread and takes no slot
+from a pool; all compute the same FP32 operations, so radiance, signatures and ray counts must be equal bit for bit."""
 import numpy as np
 import pytest
 
@@ -33,18 +34,19 @@ def views():
 
 @pytest.mark.parametrize("scene", ["soup", "spheres", "placed"])
 @pytest.mark.parametrize("width,height,spp", SIZES)
-def test_pooled_walks_equal_the_megakernel(views, scene, width, height, spp):
+def test_pooled_walks_equal_one_ray_per_thread(views, scene, width, height, spp):
     import torch
     g, cam = views[scene]
     cam = dict(cam, width=width, height=height)
     a = g.render(cam, spp, 4, 3, path_L=True, sig=True, mode="wavefront")
     sa = g.stats()
-    b = g.render(cam, spp, 4, 3, path_L=True, sig=True, mode="megakernel")
-    sb = g.stats()
-    assert sa["status"] == 0 and sb["status"] == 0
-    for k in ("img", "path_L", "sig"):
-        assert torch.equal(a[k], b[k]), k
-    assert (sa["extension_rays"], sa["shadow_rays"]) == (sb["extension_rays"], sb["shadow_rays"])
+    for static in (False, True):
+        b = g.render(cam, spp, 4, 3, path_L=True, sig=True, mode="megakernel", mk_static=static)
+        sb = g.stats()
+        assert sa["status"] == 0 and sb["status"] == 0
+        for k in ("img", "path_L", "sig"):
+            assert torch.equal(a[k], b[k]), (k, static)
+        assert (sa["extension_rays"], sa["shadow_rays"]) == (sb["extension_rays"], sb["shadow_rays"])
 
 
 @pytest.mark.parametrize("width,height", [(33, 1), (441, 441), (487, 799)])
