@@ -74,29 +74,40 @@ __device__ __forceinline__ uint32_t next_chunk(uint32_t* counter) {
     return ((gridDim.x * blockDim.x) >> 5) + __shfl_sync(0xFFFFFFFFu, b, 0);
 }
 
-// Chunks taken by a warp that hands their slots to its lanes one by one (the pooled walks): the current
-// chunk, how many of its slots are handed out, and the next chunk, whose claim is in flight while the
-// current one is walked.
-struct ChunkPool {
+// Slots [0, total) taken by the warps of a grid (the pooled walks).  A warp's first slots, up to one per
+// lane, are its own by its place in the grid; after those it claims, with one atomic, exactly what its idle
+// lanes need when they need it, so that no warp sits on slots while others run dry: with runs of 32 held and
+// the next run claimed ahead, warps ran dry 190 to 300 us into the 320 us walk of 2 M camera rays (1080p frame
+// 1.77 -> 1.67 ms, its two-level form 1.77 -> 1.65, 128 x 128 box 283 -> 256 us; claiming ahead except for the
+// last 32, 64, 96, 128, 192 slots per warp: 1.744, 1.712, 1.697, 1.685, 1.676).  `counter` is zero at launch.
+struct SlotPool {
     uint32_t* counter;
-    uint32_t c, used = 0, n_warps;
-    uint32_t raw;             // lane 0: the claim of the next chunk (consumed by a shuffle when needed)
-    uint32_t c_all;
-    __device__ __forceinline__ ChunkPool(uint32_t* ctr, uint32_t chunks)
-        : counter(ctr), c(first_chunk()), n_warps((gridDim.x * blockDim.x) >> 5), raw(0u), c_all(chunks) {
-        claim();
+    uint32_t total, first;               // slots, and those that need no claim
+    uint32_t own, own_end;               // the warp's first slots
+    uint32_t seen;                       // slots up to here are taken for certain
+    __device__ __forceinline__ SlotPool(uint32_t* ctr, uint32_t n) : counter(ctr), total(n), seen(0u) {
+        const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
+        const uint32_t size = min(32u, (n + n_warps - 1u) / n_warps);
+        own = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * size;
+        own_end = own + size;
+        first = n_warps * size;
     }
-    // no atomic when the chunks do not outnumber the warps: every claim would come back beyond the end
-    __device__ __forceinline__ void claim() {
-        if (c_all > n_warps && lane_id() == 0u) raw = atomicAdd(counter, 1u);
-    }
-    __device__ __forceinline__ uint32_t peek() const {
-        return c_all > n_warps ? n_warps + __shfl_sync(0xFFFFFFFFu, raw, 0) : c_all;
-    }
-    __device__ __forceinline__ void advance(uint32_t next) {
-        c = next;
-        used = 0u;
-        claim();
+    __device__ __forceinline__ bool more() const { return seen < total; }
+    // This lane's slot of those handed to the lanes of `idle` (all 32 lanes call it), or >= total.
+    __device__ __forceinline__ uint32_t take(uint32_t idle) {
+        const uint32_t k = (uint32_t)__popc(idle), rank = (uint32_t)__popc(idle & ((1u << lane_id()) - 1u));
+        uint32_t j;
+        if (seen == 0u) {                // the first call finds every lane idle
+            j = own + rank < own_end ? own + rank : total;
+            seen = first;
+        } else {
+            uint32_t b = 0u;
+            if (lane_id() == 0u) b = atomicAdd(counter, k);
+            b = first + __shfl_sync(0xFFFFFFFFu, b, 0);
+            j = b + rank;
+            seen = b + k;
+        }
+        return ((idle >> lane_id()) & 1u) ? j : total;
     }
 };
 

@@ -137,12 +137,12 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_ex
     const float4* __restrict__ qo = b == 0u ? nullptr : w.q_o[in];
     const float4* __restrict__ qd = w.q_d[in];
     float2* __restrict__ hit = w.hit;
-    const uint32_t chunks = (n + 31u) / 32u;
     if constexpr (SK == 0 && !CNT) {
-        ChunkPool q(&w.bc[b].claim, chunks);
-        pool_walk<INST>(src.scene(0), q, chunks, n, 0u, ExtendIo<Src, INST>{src, qo, qd, hit, w.hit_inst, base});
+        SlotPool q(&w.bc[b].claim, n);
+        pool_walk<INST>(src.scene(0), q, n, ExtendIo<Src, INST>{src, qo, qd, hit, w.hit_inst, base});
     } else {       // single-level, in lockstep
         typename std::conditional<CNT, TravCount, NoCount>::type cnt;
+        const uint32_t chunks = (n + 31u) / 32u;
         for (uint32_t c = first_chunk(); c < chunks; c = next_chunk(&w.bc[b].claim)) {
             const uint32_t j = c * 32u + lane_id();
             if (j >= n) continue;
@@ -479,13 +479,13 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
         trace_groups<Src, SIG, INST, ADJ>(src, w, a, in, b, n_ext, n_shd, G);
         return;
     }
-    const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
     if constexpr (!CNT) {
-        ChunkPool q(&w.bc[b].claim, c_all);
-        pool_walk<INST>(src.scene(0), q, c_ext, n_ext, n_shd,
+        SlotPool q(&w.bc[b].claim, n_ext + n_shd);
+        pool_walk<INST>(src.scene(0), q, n_ext,
                         TraceIo<Src, SIG, INST, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, w.hit_inst, base}, w, a, b});
     } else {       // counting (single-level, no signatures), in lockstep
         TravCount cc, ca;
+        const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
         uint32_t c = first_chunk();
         for (; c < c_ext; c = next_chunk(&w.bc[b].claim)) {
             const uint32_t j = c * 32u + lane_id();

@@ -15,8 +15,7 @@
 // a lane) takes 16 cycles of the L1 data path whether 20 or 32 lanes need it: that path is busy 76% of
 // the time (issue 58%, long-scoreboard stalls for the rest) in the launch of bounce 1 at 1080p on 1.15 M
 // triangles.  Against the lockstep walk: extension rays 15.4 -> 22 lanes per node step, bounce 1 9.5 ->
-// 19.7, 683 -> 585 us; the 1080p frame 1.96 -> 1.73 ms, a 1.07 M-triangle terrain at 2560 x 1440, 3 samples,
-// depth 8 13.04 -> 10.63 ms.
+// 19.7, 683 -> 585 us.
 #pragma once
 #include "pt_common.cuh"
 
@@ -24,11 +23,12 @@ namespace pt {
 
 constexpr uint32_t kDone = 0xFFFFFFFFu;    // no subtree left (never a leaf reference: triangles < 2^28)
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
-// 12 and 12 measured best of {8..24} x {4..16} lanes: fewer node lanes waste L1 cycles, more make the
-// loop leave its node steps too often (20 and 8: 1.887 ms per frame against 1.870 at 16 and 8); a refill
-// costs about 150 instructions for the whole warp.
-constexpr uint32_t kNodeLanes = 12;
-constexpr uint32_t kIdleLanes = 12;
+// 8 and 20 measured best over the frames of {8, 10, 12} x {8, 12, 16, 20} lanes (1080p 1.600 ms against 1.648 at
+// 12 and 12, 1.658 at 12 and 8; the terrain 9.61 against 9.87 and 10.18): fewer node lanes waste L1 cycles, more
+// make the loop leave its node steps too often; a refill costs some 150 instructions and a claim for the
+// whole warp, however few lanes it serves.
+constexpr uint32_t kNodeLanes = 8;
+constexpr uint32_t kIdleLanes = 20;
 
 // Original id of a hit, looked up only to decide ties: the triangle's, in a two-level scene offset by the
 // instance's first id.
@@ -175,55 +175,25 @@ struct Walker {
 // far below 2^31: a path's records take 180 bytes).
 constexpr uint32_t kAnySlot = 0x80000000u;
 
-// Hand out the next slots of the pool to the lanes of `idle` (all 32 lanes call it): this lane's slot, or
-// kNoSlot.  Chunks [0, c_ext) cover the n_ext extension rays, the rest the n_shd shadow rays.
-__device__ __forceinline__ uint32_t pool_take(ChunkPool& q, uint32_t c_ext, uint32_t n_ext, uint32_t n_shd,
-                                              uint32_t idle) {
-    const uint32_t lane = lane_id(), k = (uint32_t)__popc(idle), rank = (uint32_t)__popc(idle & ((1u << lane) - 1u));
-    const uint32_t avail = 32u - q.used;
-    uint32_t c = q.c, off = q.used + rank;
-    q.used += k;
-    if (k >= avail) {          // the current chunk runs out: the rest come from the next one
-        const uint32_t nc = q.peek();
-        if (rank >= avail) {
-            c = nc;
-            off = rank - avail;
-        }
-        q.advance(nc);
-        q.used = k - avail;
-    }
-    uint32_t j = kNoSlot;
-    if ((idle >> lane) & 1u) {
-        if (c < c_ext) {
-            const uint32_t i = c * 32u + off;
-            if (i < n_ext) j = i;
-        } else if (c < q.c_all) {
-            const uint32_t i = (c - c_ext) * 32u + off;
-            if (i < n_shd) j = i | kAnySlot;
-        }
-    }
-    return j;
-}
-
+// The pool's slots [0, n_ext) are the extension rays, [n_ext, q.total) the shadow rays.
 template <bool INST, class Io>
-__device__ __forceinline__ void pool_walk(const DevScene& s, ChunkPool& q, uint32_t c_ext, uint32_t n_ext,
-                                          uint32_t n_shd, const Io& io) {
+__device__ __forceinline__ void pool_walk(const DevScene& s, SlotPool& q, uint32_t n_ext, const Io& io) {
     Walker<INST> k(s);
     typename Walker<INST>::Stack stk;
     uint32_t slot = kNoSlot, steps = 0;
     while (true) {
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, k.ref == kDone);
         const bool all = idle == 0xFFFFFFFFu;
-        if (all || ((uint32_t)__popc(idle) >= kIdleLanes && q.c < q.c_all)) {
+        if (all || ((uint32_t)__popc(idle) >= kIdleLanes && q.more())) {
             if (k.ref == kDone && slot != kNoSlot) {
                 io.emit(slot, k.tbest, k.best, k.binst);
                 slot = kNoSlot;
             }
-            if (q.c >= q.c_all) break;
-            const uint32_t j = pool_take(q, c_ext, n_ext, n_shd, idle);
-            if (j != kNoSlot) {
-                slot = j;
-                io.fetch(j, k.o, k.d, k.tbest, k.best, k.nodes, k.tris);
+            if (!q.more()) break;
+            const uint32_t j = q.take(idle);
+            if (j < q.total) {
+                slot = j < n_ext ? j : (j - n_ext) | kAnySlot;
+                io.fetch(slot, k.o, k.d, k.tbest, k.best, k.nodes, k.tris);
                 k.begin(s);
             }
             steps = 0;
