@@ -50,6 +50,7 @@ struct ExtendIo {
     float2* __restrict__ hit;
     uint32_t* __restrict__ hit_inst;
     uint64_t base;
+    __device__ __forceinline__ DevScene scene() const { return src.scene(0u); }
     __device__ __forceinline__ void fetch(uint32_t j, float3& o, float3& d, float& tbest, uint32_t& best,
                                           const float4*& nodes, const float4*& tris) const {
         const float4 d4 = __ldcs(&qd[j]);
@@ -77,6 +78,7 @@ struct TraceIo {
     const WfBuffers& w;
     const AdjBuffers& a;
     uint32_t b;
+    __device__ __forceinline__ DevScene scene() const { return ext.scene(); }
     __device__ __forceinline__ void fetch(uint32_t slot, float3& o, float3& d, float& tbest, uint32_t& best,
                                           const float4*& nodes, const float4*& tris) const {
         if (!(slot & kAnySlot)) {
@@ -128,8 +130,9 @@ constexpr int trace_blocks(bool inst, bool pooled) { return inst ? 4 : pooled ? 
 // Extend: closest hit of every active ray (scene-intersection stage); hit records per queue slot.
 // SK > 0: the walks keep their top SK stack entries in dynamic shared memory (single-level only).
 // CNT: count the walks' node visits and triangle tests into the scene's traversal counters.
-template <class Src, bool INST, int SK = 0, bool CNT = false>
-__global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_extend(Src src, WfBuffers w, int in, uint32_t b) {
+template <class Src, bool INST, int SK = 0, bool CNT = false, bool SHARE = false>
+__global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_extend(
+    const __grid_constant__ Src src, const __grid_constant__ WfBuffers w, int in, uint32_t b) {
     stage_prologue();
     const uint32_t n = min(w.bc[b].active, w.capacity);
     if (n == 0u) return;       // an emptied queue: no claims (the same for every thread)
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, SK == 0 && !CNT)) k_ex
     float2* __restrict__ hit = w.hit;
     if constexpr (SK == 0 && !CNT) {
         SlotPool q(&w.bc[b].claim, n);
-        pool_walk<INST>(src.scene(0), q, n, ExtendIo<Src, INST>{src, qo, qd, hit, w.hit_inst, base});
+        pool_walk<INST, SHARE>(src.scene(0), q, n, ExtendIo<Src, INST>{src, qo, qd, hit, w.hit_inst, base});
     } else {       // single-level, in lockstep
         typename std::conditional<CNT, TravCount, NoCount>::type cnt;
         const uint32_t chunks = (n + 31u) / 32u;
@@ -383,7 +386,8 @@ __global__ void __launch_bounds__(256) k_shadow(Src src, WfBuffers w, uint32_t b
 // group's first lane writes the result exactly as the one-lane form does.
 constexpr uint32_t kCoopMinLanes = 2u;
 
-template <class Src, bool SIG, bool INST, bool ADJ>
+// SHARE only sets the two kernels' copies apart: ptxas 13.0 crashes on one function called by both.
+template <class Src, bool SIG, bool INST, bool ADJ, bool SHARE>
 __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, const AdjBuffers& a, int in,
                                              uint32_t b, uint32_t n_ext, uint32_t n_shd, uint32_t G) {
     const uint64_t base = src.base();
@@ -459,8 +463,9 @@ __device__ __noinline__ void trace_groups(const Src& src, const WfBuffers& w, co
 // instead of running after a stage boundary.
 // ADJ: the adjoint replay's variant, whose shadow walks mark the vertex record's NEE sample visible
 // (flag 2 of record 3 of bounce b - 1) instead of adding a contribution.
-template <class Src, bool SIG, bool INST, bool CNT = false, bool ADJ = false>
-__global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src, WfBuffers w, AdjBuffers a, int in, uint32_t b) {
+template <class Src, bool SIG, bool INST, bool CNT = false, bool ADJ = false, bool SHARE = false>
+__global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(
+    const __grid_constant__ Src src, const __grid_constant__ WfBuffers w, const __grid_constant__ AdjBuffers a, int in, uint32_t b) {
     stage_prologue();
     const uint32_t n_ext = min(w.bc[b].active, w.capacity), n_shd = min(w.bc[b].shadow, w.capacity);
     if (n_ext + n_shd == 0u) return;       // the same for every thread
@@ -476,13 +481,13 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(Src src
         if (G < kCoopMinLanes) G = 1u;
     }
     if (G > 1u) {
-        trace_groups<Src, SIG, INST, ADJ>(src, w, a, in, b, n_ext, n_shd, G);
+        trace_groups<Src, SIG, INST, ADJ, SHARE>(src, w, a, in, b, n_ext, n_shd, G);
         return;
     }
     if constexpr (!CNT) {
         SlotPool q(&w.bc[b].claim, n_ext + n_shd);
-        pool_walk<INST>(src.scene(0), q, n_ext,
-                        TraceIo<Src, SIG, INST, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, w.hit_inst, base}, w, a, b});
+        pool_walk<INST, SHARE>(src.scene(0), q, n_ext,
+                               TraceIo<Src, SIG, INST, ADJ>{{src, w.q_o[in], w.q_d[in], w.hit, w.hit_inst, base}, w, a, b});
     } else {       // counting (single-level, no signatures), in lockstep
         TravCount cc, ca;
         const uint32_t c_ext = (n_ext + 31u) / 32u, c_all = c_ext + (n_shd + 31u) / 32u;
@@ -650,6 +655,7 @@ cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w
     if (p.count_trav) return launch_k(l, 0, k_extend<SingleSrc, false, 0, true>, src, w, in, bounce);
     if (p.short_stack)
         return launch_k(l, stack_smem_bytes(kShortStack, l.block), k_extend<SingleSrc, false, kShortStack>, src, w, in, bounce);
+    if (p.share) return launch_k(l, 0, k_extend<SingleSrc, false, 0, false, true>, src, w, in, bounce);
     return launch_k(l, 0, k_extend<SingleSrc, false>, src, w, in, bounce);
 }
 
@@ -755,6 +761,7 @@ cudaError_t launch_trace(const Launch& l, const DevScene& s, const RenderParams&
     }
     if (p.count_trav && !w.sig) return launch_k(l, 0, k_trace<SingleSrc, false, false, true>, src, w, a, in, bounce);
     if (w.sig) return launch_k(l, 0, k_trace<SingleSrc, true, false>, src, w, a, in, bounce);
+    if (p.share) return launch_k(l, 0, k_trace<SingleSrc, false, false, false, false, true>, src, w, a, in, bounce);
     return launch_k(l, 0, k_trace<SingleSrc, false, false>, src, w, a, in, bounce);
 }
 
@@ -762,6 +769,7 @@ cudaError_t launch_trace_adj(const Launch& l, const DevScene& s, const RenderPar
                              const AdjBuffers& a, int in, uint32_t bounce) {
     SingleSrc src{s, DevCamera{}, p};
     if (s.tlas) return launch_k(l, 0, k_trace<SingleSrc, false, true, false, true>, src, w, a, in, bounce);
+    if (p.share) return launch_k(l, 0, k_trace<SingleSrc, false, false, false, true, true>, src, w, a, in, bounce);
     return launch_k(l, 0, k_trace<SingleSrc, false, false, false, true>, src, w, a, in, bounce);
 }
 

@@ -25,7 +25,7 @@
 namespace pt {
 pt_status static_set_error(pt_status s, const char* msg);
 pt_status static_prepare(pt_scene* sc, const pt_camera* cam, const pt_render_opts* opts, DevScene* view,
-                         DevCamera* dc, pt_render_opts* o_out, int* device);
+                         DevCamera* dc, pt_render_opts* o_out, int* device, uint32_t* share);
 bool static_is_device_ptr(const void* p);
 }  // namespace pt
 
@@ -87,7 +87,8 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
     pt::DevCamera dc;
     pt_render_opts o;
     int device = 0;
-    pt_status s = pt::static_prepare(scene, cam, opts, &ds, &dc, &o, &device);
+    uint32_t share = 0;
+    pt_status s = pt::static_prepare(scene, cam, opts, &ds, &dc, &o, &device, &share);
     if (s != PT_OK) return s;
     if (o.mode != PT_MODE_WAVEFRONT)
         return pt::static_set_error(PT_ERR_INVALID_ARG, "this entry point renders with the wavefront only (opts->mode)");
@@ -176,6 +177,7 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
     for (uint64_t w0 = 0; w0 < n_paths; w0 += cap) {
         const uint32_t n = (uint32_t)std::min<uint64_t>(cap, n_paths - w0);
         p.path_begin = w0;
+        p.share = fused ? share : 0u;
         p.ex = dc.ex;
         p.ey = dc.ey;
         p.ez = dc.ez;

@@ -59,6 +59,7 @@ struct RenderParams {
     uint32_t mis = 0;             // 1: NEE and BSDF-sampled light hits combined by the power heuristic
     uint32_t short_stack = 0;     // 1: single-level walks keep their top stack entries in shared memory
     float ex = 0.f, ey = 0.f, ez = 0.f;   // the camera's eye: the origin of every ray of bounce 0
+    uint32_t share = 0;           // 1: the ends of the trace launches share walks (pool_drain)
     uint32_t count_trav = 0;      // 1: single-level walks count visited nodes and tested triangles
 };
 

@@ -62,3 +62,34 @@ def test_pooled_replay_equals_the_separate_order(views, width, height):
     for x, y in ((ga, ha), (ge, he)):
         assert float((x - y).abs().max()) <= 1e-5 * max(float(y.abs().max()), 1e-30)
     assert np.isfinite(float(ga.sum()))
+
+
+@pytest.fixture(scope="module")
+def large():
+    import paper_2605_27323_gb300 as pt
+    sc = scenes.spheres_scene(seed=7, n_spheres=30, level=4, ground_quads=160, extent=12.0)
+    g = pt.Scene.from_dict(sc)
+    assert g.info()["n_nodes"] >= 1 << 16
+    return g, sc["camera"]
+
+
+@pytest.mark.parametrize("width,height,spp", [(33, 1, 1), (311, 313, 1), (441, 441, 1), (487, 799, 1), (523, 397, 3)])
+def test_shared_last_walks_equal_one_ray_per_thread(large, width, height, spp):
+    """Trees of 2^16 nodes and more: the last walks of a trace launch are shared among a warp's lanes (renders
+    without signatures).  The hit of a shared walk is the smallest (t, original id), that of a walk in one lane."""
+    import torch
+    g, cam = large
+    cam = dict(cam, width=width, height=height)
+    a = g.render(cam, spp, 4, 3, path_L=True, mode="wavefront")
+    sa = g.stats()
+    b = g.render(cam, spp, 4, 3, path_L=True, mode="megakernel", mk_static=True)
+    sb = g.stats()
+    assert sa["status"] == 0 and sb["status"] == 0
+    for k in ("img", "path_L"):
+        assert torch.equal(a[k], b[k]), k
+    assert (sa["extension_rays"], sa["shadow_rays"]) == (sb["extension_rays"], sb["shadow_rays"])
+    grad = torch.ones((height, width, 3), device="cuda") / (width * height)
+    ga, ge = g.backward(cam, spp, 4, 3, grad)
+    ha, he = g.backward(cam, spp, 4, 3, grad, separate_shadow=True)
+    for x, y in ((ga, ha), (ge, he)):
+        assert float((x - y).abs().max()) <= 1e-5 * max(float(y.abs().max()), 1e-30)
