@@ -188,9 +188,9 @@ struct pt_scene {
     unsigned long long* rays() const { return hist() + 128; }
 
     // Large trees: the ends of the fused order's trace launches share walks (pool_drain).  The 1080p frame of 1.15 M
-    // triangles (0.6 M nodes) 1.602 -> 1.548 ms, of 0.22 M triangles 1.442 -> 1.429; 95 k triangles even; the
-    // 36-triangle box, whose walks are over in a few steps, 249 -> 270 us.
-    static constexpr uint64_t kShareNodes = 1u << 16;
+    // triangles (0.6 M nodes) 1.602 -> 1.548 ms, of 0.22 M triangles 1.442 -> 1.429, four 720p frames of 95 k triangles
+    // 2.187 -> 2.148; the 36-triangle box, whose walks are over in a few steps, 249 -> 270 us.
+    static constexpr uint64_t kShareNodes = 1u << 14;
     uint32_t shares_walks() const { return !instanced && n_nodes >= kShareNodes ? 1u : 0u; }
     uint32_t* status() const { return counters.as<uint32_t>() + pt::kStatusWord; }
     pt_status ensure_counters() { return counters.ensure(pt::kCounterBytes); }

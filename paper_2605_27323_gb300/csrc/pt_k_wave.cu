@@ -385,6 +385,10 @@ __global__ void __launch_bounds__(256) k_shadow(Src src, WfBuffers w, uint32_t b
 // one shadow ray, per claim (trace_closest_group / trace_any_group, or their two-level forms); the
 // group's first lane writes the result exactly as the one-lane form does.
 constexpr uint32_t kCoopMinLanes = 2u;
+// Groups of two lanes only below this many walks: from there on the pooled walk is the faster one (the launch of
+// 56 k walks at bounce 4 of a 1080p frame: 1.547 -> 1.510 ms for the frame, its two-level form 1.608 -> 1.585, four 720p
+// frames 2.242 -> 2.187); in the grids of small images, sized to their queues, groups of two are.
+constexpr uint32_t kPairMaxWalks = 1u << 15;
 
 // SHARE only sets the two kernels' copies apart: ptxas 13.0 crashes on one function called by both.
 template <class Src, bool SIG, bool INST, bool ADJ, bool SHARE>
@@ -471,14 +475,14 @@ __global__ void __launch_bounds__(256, trace_blocks(INST, !CNT)) k_trace(
     if (n_ext + n_shd == 0u) return;       // the same for every thread
     const uint64_t base = src.base();
     // Lanes per walk: 1 while the walks fill the grid; once they are few (the sparse late bounces),
-    // the largest power of two G <= 32 with walks x G <= the grid's threads (cooperative walks; the
+    // the largest power of two G <= 32 with walks x G <= the grid's threads (cooperative walks, see kPairMaxWalks; the
     // counting instantiations keep the one-lane walk their counts describe).
     // The same for every thread: the counts are fixed during the launch.
     uint32_t G = 1u;
     if constexpr (!CNT) {
         const uint64_t threads = (uint64_t)gridDim.x * blockDim.x;
         while (G < 32u && (uint64_t)(n_ext + n_shd) * (2u * G) <= threads) G *= 2u;
-        if (G < kCoopMinLanes) G = 1u;
+        if (G < kCoopMinLanes || (G < 4u && n_ext + n_shd >= kPairMaxWalks)) G = 1u;
     }
     if (G > 1u) {
         trace_groups<Src, SIG, INST, ADJ, SHARE>(src, w, a, in, b, n_ext, n_shd, G);

@@ -69,13 +69,13 @@ def large():
     import paper_2605_27323_gb300 as pt
     sc = scenes.spheres_scene(seed=7, n_spheres=30, level=4, ground_quads=160, extent=12.0)
     g = pt.Scene.from_dict(sc)
-    assert g.info()["n_nodes"] >= 1 << 16
+    assert g.info()["n_nodes"] >= 1 << 14
     return g, sc["camera"]
 
 
 @pytest.mark.parametrize("width,height,spp", [(33, 1, 1), (311, 313, 1), (441, 441, 1), (487, 799, 1), (523, 397, 3)])
 def test_shared_last_walks_equal_one_ray_per_thread(large, width, height, spp):
-    """Trees of 2^16 nodes and more: the last walks of a trace launch are shared among a warp's lanes (renders
+    """Trees of 2^14 nodes and more: the last walks of a trace launch are shared among a warp's lanes (renders
     without signatures).  The hit of a shared walk is the smallest (t, original id), that of a walk in one lane."""
     import torch
     g, cam = large
