@@ -1457,7 +1457,8 @@ pt_status pt_trace_closest(pt_scene* sc, const float* d_rays, uint32_t n, float*
     PT_TRY(set_device(sc));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     sc->last_stream = st;
-    PT_CUDA(pt::launch_trace_closest(launch_for(sc, pt::K_EXTEND, 0, 256, st, n), sc->view(), d_rays, n, d_t, d_prim));
+    PT_CUDA(pt::launch_trace_closest(launch_for(sc, pt::K_EXTEND, 0, 256, st, n), sc->view(), d_rays, n, d_t, d_prim,
+                                     sc->shares_walks() != 0u));
     return PT_OK;
 }
 

@@ -111,6 +111,28 @@ struct SlotPool {
     }
 };
 
+// The same slots dealt out without a counter, runs of 32 to the warps in turn (closest-hit queries, which keep no
+// state between calls: calls on one scene may overlap on several streams).
+struct DealtPool {
+    uint32_t total, n_warps, warp;
+    uint32_t used = 0u;                  // of the warp's own sequence
+    __device__ __forceinline__ explicit DealtPool(uint32_t n) : total(n) {
+        n_warps = (gridDim.x * blockDim.x) >> 5;
+        warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    }
+    __device__ __forceinline__ uint32_t slot(uint32_t i) const {
+        const uint64_t j = ((uint64_t)(i >> 5) * n_warps + warp) * 32u + (i & 31u);
+        return j < total ? (uint32_t)j : total;
+    }
+    __device__ __forceinline__ bool more() const { return slot(used) < total; }
+    __device__ __forceinline__ uint32_t take(uint32_t idle) {
+        const uint32_t rank = (uint32_t)__popc(idle & ((1u << lane_id()) - 1u));
+        const uint32_t j = slot(used + rank);
+        used += (uint32_t)__popc(idle);
+        return ((idle >> lane_id()) & 1u) ? j : total;
+    }
+};
+
 __device__ __forceinline__ void warp_add_u64(unsigned long long* dst, unsigned long long v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
     if (lane_id() == 0 && v) atomicAdd(dst, v);

@@ -1,6 +1,9 @@
 // pt_k_util.cu -- material updates, closest-hit queries, the random-number probe, and the
 // occupancy table used to size persistent grids.
+#include <algorithm>
+
 #include "pt_common.cuh"
+#include "pt_pool.cuh"
 
 namespace pt {
 
@@ -16,16 +19,35 @@ __global__ void k_set_materials(DevMat* mats, uint32_t n, const float* albedo, c
     if (emission) mats[m].emission = emission[m];
 }
 
+// Closest hits of n rays of 8 floats (origin, -, direction, -), by pooled walks.  The caller's rays need no more than
+// float alignment.
 template <bool INST>
-__global__ void __launch_bounds__(256) k_trace_closest(DevScene s, const float* __restrict__ rays, uint32_t n,
-                                                       float* __restrict__ t, int32_t* __restrict__ prim) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+struct QueryIo {
+    const DevScene& s;
+    const float* __restrict__ rays;
+    float* __restrict__ t;
+    int32_t* __restrict__ prim;
+    __device__ __forceinline__ DevScene scene() const { return s; }
+    __device__ __forceinline__ void fetch(uint32_t i, float3& o, float3& d, float& tbest, uint32_t& best,
+                                          const float4*&, const float4*&) const {
         const float* r = rays + 8 * (size_t)i;
-        Hit h = trace_closest<INST>(s, f3(r[0], r[1], r[2]), f3(r[4], r[5], r[6]));
-        t[i] = h.t;
-        prim[i] = h.tri == kMiss ? -1 : (int32_t)h.prim;
+        o = f3(__ldg(r), __ldg(r + 1), __ldg(r + 2));
+        d = f3(__ldg(r + 4), __ldg(r + 5), __ldg(r + 6));
+        tbest = __int_as_float(0x7f800000);
+        best = kMiss;
     }
+    __device__ __forceinline__ void emit(uint32_t i, float th, uint32_t tri, uint32_t inst) const {
+        t[i] = th;
+        prim[i] = tri == kMiss ? -1 : (int32_t)pool_id<INST>(s, s.tris, tri, inst);
+    }
+};
+
+template <bool INST, bool SHARE>
+__global__ void __launch_bounds__(256, INST ? 4 : 5) k_trace_closest(const __grid_constant__ DevScene s,
+                                                                     const float* __restrict__ rays, uint32_t n,
+                                                                     float* __restrict__ t, int32_t* __restrict__ prim) {
+    DealtPool q(n);
+    pool_walk<INST, SHARE>(s, q, n, QueryIo<INST>{s, rays, t, prim});
 }
 
 __global__ void k_debug_rng(uint64_t seed, const uint32_t* px, const uint32_t* sm, const uint32_t* bo,
@@ -43,9 +65,15 @@ cudaError_t launch_set_materials(cudaStream_t st, DevMat* mats, uint32_t n, cons
 }
 
 cudaError_t launch_trace_closest(const Launch& l, const DevScene& s, const float* rays, uint32_t n, float* t,
-                                 int32_t* prim) {
-    if (s.tlas) k_trace_closest<true><<<l.grid, l.block, 0, l.st>>>(s, rays, n, t, prim);
-    else k_trace_closest<false><<<l.grid, l.block, 0, l.st>>>(s, rays, n, t, prim);
+                                 int32_t* prim, bool share) {
+    // a slot of the pool has 31 bits
+    for (uint64_t i = 0; i < n; i += 1u << 30) {
+        const uint32_t m = (uint32_t)std::min<uint64_t>(n - i, 1u << 30);
+        const float* r = rays + 8 * i;
+        if (s.tlas) k_trace_closest<true, false><<<l.grid, l.block, 0, l.st>>>(s, r, m, t + i, prim + i);
+        else if (share) k_trace_closest<false, true><<<l.grid, l.block, 0, l.st>>>(s, r, m, t + i, prim + i);
+        else k_trace_closest<false, false><<<l.grid, l.block, 0, l.st>>>(s, r, m, t + i, prim + i);
+    }
     return cudaGetLastError();
 }
 

@@ -321,8 +321,8 @@ __device__ __noinline__ void pool_drain(const Io& io, DrainShared& sh, uint32_t 
 
 // The pool's slots [0, n_ext) are the extension rays, [n_ext, q.total) the shadow rays.
 // SHARE: the end of the pool is walked by pool_drain.
-template <bool INST, bool SHARE, class Io>
-__device__ __forceinline__ void pool_walk(const DevScene& s, SlotPool& q, uint32_t n_ext, const Io& io) {
+template <bool INST, bool SHARE, class Pool, class Io>
+__device__ __forceinline__ void pool_walk(const DevScene& s, Pool& q, uint32_t n_ext, const Io& io) {
     __shared__ DrainShared sh[SHARE ? 8 : 1];
     Walker<INST> k(s);
     typename Walker<INST>::Stack stk;
@@ -349,7 +349,7 @@ __device__ __forceinline__ void pool_walk(const DevScene& s, SlotPool& q, uint32
             if (!q.more()) break;
             const uint32_t j = q.take(idle);
             if (j < q.total) {
-                slot = j < n_ext ? j : (j - n_ext) | kAnySlot;
+                slot = j < n_ext ? j : ((j - n_ext) | kAnySlot);
                 io.fetch(slot, k.o, k.d, k.tbest, k.best, k.nodes, k.tris);
                 k.begin(s);
             }

@@ -227,7 +227,7 @@ class Scene:
         o = torch.as_tensor(o, dtype=torch.float32, device="cuda").reshape(-1, 3)
         d = torch.as_tensor(d, dtype=torch.float32, device="cuda").reshape(-1, 3)
         n = o.shape[0]
-        rays = torch.zeros((n, 8), device="cuda", dtype=torch.float32)
+        rays = torch.empty((n, 8), device="cuda", dtype=torch.float32)      # lanes 3 and 7 are not read
         rays[:, 0:3] = o
         rays[:, 4:7] = d
         t = torch.empty(n, device="cuda", dtype=torch.float32)

@@ -93,3 +93,38 @@ def test_shared_last_walks_equal_one_ray_per_thread(large, width, height, spp):
     ha, he = g.backward(cam, spp, 4, 3, grad, separate_shadow=True)
     for x, y in ((ga, ha), (ge, he)):
         assert float((x - y).abs().max()) <= 1e-5 * max(float(y.abs().max()), 1e-30)
+
+
+def _query(g, rays, n):
+    import ctypes as C
+
+    import torch
+
+    from paper_2605_27323_gb300 import capi
+    t = torch.empty(n, device="cuda")
+    prim = torch.empty(n, device="cuda", dtype=torch.int32)
+    capi.check(capi.load().pt_trace_closest(g.h, C.c_void_p(rays), n, C.c_void_p(t.data_ptr()), C.c_void_p(prim.data_ptr()),
+                                            C.c_void_p(torch.cuda.current_stream().cuda_stream)))
+    return t, prim
+
+
+@pytest.mark.parametrize("scene", ["soup", "placed", "large"])
+@pytest.mark.parametrize("n", [1, 31, 33, 194559, 194561, 400003])
+def test_pooled_queries(views, large, scene, n):
+    """Closest-hit queries at the edges of a warp's runs and of the grid, with rays at float alignment only: each
+    ray's hit is that of a query of a few rays (a run of its own warp), whatever its place."""
+    import torch
+    g = large[0] if scene == "large" else views[scene][0]
+    o, d = scenes.random_rays(n, seed=n, spread=1.5)
+    rays = torch.zeros(8 * n + 1, device="cuda")
+    r = rays[1:].view(n, 8)
+    r[:, 0:3] = torch.as_tensor(o * (1.0 if scene == "soup" else 4.0), dtype=torch.float32, device="cuda")
+    r[:, 4:7] = torch.as_tensor(d, dtype=torch.float32, device="cuda")
+    t, prim = _query(g, r.data_ptr(), n)
+    at = sorted({0, n - 1, n // 2, n // 3, 7 * n // 8})
+    for i in at:
+        m = min(n - i, 5)
+        few = r[i:i + m].clone()
+        t1, p1 = _query(g, few.data_ptr(), m)
+        assert torch.equal(t[i:i + m], t1) and torch.equal(prim[i:i + m], p1), i
+    assert bool(((prim >= 0) == torch.isfinite(t)).all())
