@@ -181,9 +181,9 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
         p.ex = dc.ex;
         p.ey = dc.ey;
         p.ez = dc.ez;
-        pt::Launch le = persistent(per_extend, n), ls = persistent(per_shade, n);
+        pt::Launch le = persistent(per_extend, 4ull * n), ls = persistent(per_shade, n);
         const pt::Launch lw = persistent(per_shadow, n);
-        pt::Launch lt = persistent(per_trace, 2ull * n), lr = plain(n / spp);
+        pt::Launch lt = persistent(per_trace, 8ull * n), lr = plain(n / spp);
         // fused: the stage kernels are programmatic dependents of the kernel before them, as in pt_render
         le.pdl = ls.pdl = lt.pdl = lr.pdl = fused && n_keys == 0;
         if ((e = pt::launch_raygen(plain(n), dc, p, n, w)) != cudaSuccess) return cuda_fail(e, "raygen");
