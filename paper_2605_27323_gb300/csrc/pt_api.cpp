@@ -411,7 +411,9 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
         p.ez = cam.ez;
         size_t ev = 0;
         PT_TRY(sc->ev_begin(ST_RAYGEN, st, ev));
-        PT_CUDA(pt::launch_raygen(simple_launch(sc, st, n), cam, p, n, w));
+        pt::Launch lg = simple_launch(sc, st, n);
+        lg.pdl = kStagePdl;
+        PT_CUDA(pt::launch_raygen(lg, cam, p, n, w, w0 == 0));
         PT_TRY(sc->ev_end(ev, st));
         sc->launches += 1;
         // fused: each bounce's extend launch also walks the shadow rays the previous shading cast
@@ -479,10 +481,12 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
             }
         }
         PT_TRY(sc->ev_begin(ST_REDUCE, st, ev));
-        if (accum)
-            PT_CUDA(pt::launch_accumulate(simple_launch(sc, st, n / p.spp), reinterpret_cast<const float*>(w.L), 4,
+        if (accum) {
+            pt::Launch la = simple_launch(sc, st, n / p.spp);
+            la.pdl = kStagePdl;
+            PT_CUDA(pt::launch_accumulate(la, reinterpret_cast<const float*>(w.L), 4,
                                           w0 / p.spp, n / p.spp, p.spp, accum, count, img, &w));
-        else {
+        } else {
             pt::Launch lr = simple_launch(sc, st, n / p.spp);
             lr.pdl = kStagePdl;
             PT_CUDA(pt::launch_reduce(lr, reinterpret_cast<const float*>(w.L), 4, w0 / p.spp, n / p.spp, p.spp, img, &w));
@@ -796,7 +800,8 @@ pt_status render_impl(pt_scene* sc, const pt_camera* cam, uint32_t spp, uint32_t
     sc->last_mode = o.mode;
     sc->last_paths = n_paths;
     sc->launches = 0;
-    PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
+    if (o.mode == PT_MODE_MEGAKERNEL || max_depth == 0)      // (the wavefront's ray generation clears them)
+        PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
     if (accum && sample_offset == 0) PT_CUDA(cudaMemsetAsync(accum, 0, n_pixels * 12, st));
     pt::RenderParams p;
     p.seed = seed;
@@ -1365,8 +1370,10 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
     sc->last_mode = 2;
     sc->last_paths = n_paths;
     sc->launches = 0;
-    PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
-    if (max_depth == 0 || sc->n_mats == 0) return PT_OK;
+    const bool nothing = max_depth == 0 || sc->n_mats == 0;
+    if (o.mode == PT_MODE_MEGAKERNEL || nothing)             // (the wavefront's ray generation clears them)
+        PT_CUDA(cudaMemsetAsync(sc->counters.p, 0, sc->counters.bytes, st));
+    if (nothing) return PT_OK;
     pt::RenderParams p;
     p.seed = seed;
     p.path_begin = 0;
@@ -1411,7 +1418,9 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
             pw.ez = dc.ez;
             size_t e2 = 0;
             PT_TRY(sc->ev_begin(ST_RAYGEN, st, e2));
-            PT_CUDA(pt::launch_raygen(simple_launch(sc, st, n), dc, pw, n, w));
+            pt::Launch lg = simple_launch(sc, st, n);
+            lg.pdl = kStagePdl;
+            PT_CUDA(pt::launch_raygen(lg, dc, pw, n, w, w0 == 0));
             PT_TRY(sc->ev_end(e2, st));
             // fused as the forward wavefront: each bounce's extend launch also walks the shadow rays of
             // the previous bounce (marking their records), unless the separate order is asked for

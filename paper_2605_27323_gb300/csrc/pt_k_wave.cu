@@ -18,10 +18,12 @@ namespace pt {
 // which extend and shade know at bounce 0 (16 bytes written and 2 x 16 read per path instead of 64 and
 // 32 + 64: shading the 2 M camera hits of a 1080p frame 101 -> 86 us, the frame 1.770 -> 1.753 ms).  The
 // wave's first path id is a launch argument here and is published to device memory (wave_base_dev) for the
-// kernels of the bounce loop.
+// kernels of the bounce loop.  clear: the call's first wave also zeroes the call's totals and status word (a memset
+// of their own cost a small image 3 us).
 template <class Src>
 __global__ void __launch_bounds__(256) k_raygen(Src src, uint64_t base, uint32_t n, WfBuffers w,
-                                                unsigned long long* wave_base_dev) {
+                                                unsigned long long* wave_base_dev, bool clear) {
+    stage_prologue();
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const PathLoc l = src.locate(base, i);
@@ -35,6 +37,10 @@ __global__ void __launch_bounds__(256) k_raygen(Src src, uint64_t base, uint32_t
         if (w.sig) w.sig[l.path] = 0u;
     }
     if (blockIdx.x == 0) {
+        if (clear) {
+            uint32_t* words = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(w.hist) - kHistOffset);
+            for (uint32_t k = threadIdx.x; k < (uint32_t)(kBounceOffset / 4); k += blockDim.x) words[k] = 0u;
+        }
         for (uint32_t k = threadIdx.x; k < (uint32_t)kBounceSlots; k += blockDim.x)
             w.bc[k] = BounceCounts{0u, k == 0u ? n : 0u, 0u, 0u};
         if (threadIdx.x == 0 && wave_base_dev) *wave_base_dev = base;
@@ -555,6 +561,7 @@ __global__ void __launch_bounds__(256) k_accumulate(const float* __restrict__ L,
                                                     uint64_t pixel_begin, uint64_t n_pixels, uint32_t spp,
                                                     float* __restrict__ sum, uint32_t count, float* __restrict__ img,
                                                     const BounceCounts* bc, unsigned long long* hist) {
+    stage_prologue();
     fold_counts(bc, hist);
     const float inv = 1.0f / (float)count;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -646,10 +653,10 @@ __global__ void k_scale_batch(BatchTables t, const unsigned long long* __restric
 
 // ------------------------------------------------------------------ launchers
 
-cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParams& p, uint32_t n, const WfBuffers& w) {
+cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParams& p, uint32_t n, const WfBuffers& w,
+                          bool clear) {
     SingleSrc src{DevScene{}, c, p};
-    k_raygen<SingleSrc><<<l.grid, l.block, 0, l.st>>>(src, p.path_begin, n, w, nullptr);
-    return cudaGetLastError();
+    return launch_k(l, 0, k_raygen<SingleSrc>, src, p.path_begin, n, w, (unsigned long long*)nullptr, clear);
 }
 
 cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce,
@@ -710,7 +717,7 @@ cudaError_t launch_shadow(const Launch& l, const DevScene& s, const RenderParams
 cudaError_t launch_raygen_batch(const Launch& l, const BatchTables& t, const RenderParams& p, uint64_t base, uint32_t n,
                                 const WfBuffers& w) {
     TableSrc src{t, p};
-    k_raygen<TableSrc><<<l.grid, l.block, 0, l.st>>>(src, base, n, w, t.wave_base);
+    k_raygen<TableSrc><<<l.grid, l.block, 0, l.st>>>(src, base, n, w, t.wave_base, false);
     return cudaGetLastError();
 }
 
@@ -785,9 +792,8 @@ cudaError_t launch_reduce(const Launch& l, const float* L, uint32_t stride, uint
 
 cudaError_t launch_accumulate(const Launch& l, const float* L, uint32_t stride, uint64_t pixel_begin, uint64_t n_pixels,
                               uint32_t spp, float* sum, uint32_t count, float* img, const WfBuffers* w) {
-    k_accumulate<<<l.grid, l.block, 0, l.st>>>(L, stride, pixel_begin, n_pixels, spp, sum, count, img,
-                                               w ? w->bc : nullptr, w ? w->hist : nullptr);
-    return cudaGetLastError();
+    return launch_k(l, 0, k_accumulate, L, stride, pixel_begin, n_pixels, spp, sum, count, img,
+                    w ? (const BounceCounts*)w->bc : nullptr, w ? w->hist : nullptr);
 }
 
 cudaError_t launch_copy_L(const Launch& l, const float4* L4, uint64_t n, float* out_L3) {

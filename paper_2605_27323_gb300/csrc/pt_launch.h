@@ -32,7 +32,9 @@ cudaError_t launch_debug_paths(cudaStream_t st, const DevScene& s, const DevCame
                                float* out_L);
 
 // Wavefront stages (Sec. 2.3, 3.1).  `in` selects the ping-pong queue read this bounce.
-cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParams& p, uint32_t n, const WfBuffers& w);
+// clear: the first wave of a call (its totals and status word are zeroed)
+cudaError_t launch_raygen(const Launch& l, const DevCamera& c, const RenderParams& p, uint32_t n, const WfBuffers& w,
+                          bool clear);
 cudaError_t launch_extend(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce,
                           const RenderParams& p);
 cudaError_t launch_sort(const Launch& l, const DevScene& s, const WfBuffers& w, int in, uint32_t bounce, uint32_t mode,

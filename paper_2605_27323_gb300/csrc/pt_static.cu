@@ -124,10 +124,10 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
     // scene's status word, so pt_get_stats keeps describing the scene's last pt_render call
     ds.status = reinterpret_cast<uint32_t*>(base) + pt::kStatusWord;
 
-    cudaError_t e = cudaMemsetAsync(base, 0, kHeaderBytes, st);   // counters, status word, histories
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    cudaError_t e = cudaSuccess;      // (ray generation clears the counters, status word and totals)
     if (max_depth == 0) {
-        e = cudaMemsetAsync(d_out_rgb, 0, n_pixels * 12, st);
+        e = cudaMemsetAsync(base, 0, kHeaderBytes, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_out_rgb, 0, n_pixels * 12, st);
         if (e == cudaSuccess && o.d_path_sig) e = cudaMemsetAsync(o.d_path_sig, 0, n_paths * 4, st);
         return e == cudaSuccess ? PT_OK : cuda_fail(e, "cudaMemsetAsync");
     }
@@ -186,7 +186,9 @@ extern "C" pt_status pt_render_wavefront_static(pt_scene* scene, const pt_camera
         pt::Launch lt = persistent(per_trace, 8ull * n), lr = plain(n / spp);
         // fused: the stage kernels are programmatic dependents of the kernel before them, as in pt_render
         le.pdl = ls.pdl = lt.pdl = lr.pdl = fused && n_keys == 0;
-        if ((e = pt::launch_raygen(plain(n), dc, p, n, w)) != cudaSuccess) return cuda_fail(e, "raygen");
+        pt::Launch lg = plain(n);
+        lg.pdl = le.pdl;
+        if ((e = pt::launch_raygen(lg, dc, p, n, w, w0 == 0)) != cudaSuccess) return cuda_fail(e, "raygen");
         for (uint32_t b = 0; b < max_depth; ++b) {
             const int in = (int)(b & 1u);
             if (!fused || b == 0) {          // no shadow rays are pending before the first shading
