@@ -39,7 +39,7 @@ WORKLOAD = ("procedural spheres scene: 200 level-4 icospheres + 256x256-quad gro
             "step = wavefront frame + megakernel frame + adjoint pass")
 KERNEL_SOURCES = ["paper_2605_27323_gb300/csrc/pt_k_wave.cu", "paper_2605_27323_gb300/csrc/pt_common.cuh",
                   "paper_2605_27323_gb300/csrc/pt_device.cuh", "paper_2605_27323_gb300/csrc/pt_trace.cuh",
-                  "paper_2605_27323_gb300/csrc/pt_k_mega.cu"]
+                  "paper_2605_27323_gb300/csrc/pt_pool.cuh", "paper_2605_27323_gb300/csrc/pt_k_mega.cu"]
 # Unit ceilings of the traversal kernels (per SM per cycle): 4 warp schedulers issue one warp
 # instruction each; the L1 data path moves 128 bytes.  A BVH node record is 64 bytes, a triangle
 # record 48 bytes.
@@ -52,7 +52,7 @@ BYTES_PER_UNIT = {
     "shadow": 80,      # per shadow ray: o|tmax + d|id (32 B) + contribution (16 B) read, L rw (32 B)
     "shade": 184,      # per active path: ray+tp (48) + hit (8) + L rw (32) + next ray (48) + shadow (48)
     "megakernel": 12,  # per path: radiance written (scene reads amortise to ~0 per path)
-    "raygen": 64,      # per path: ray + throughput (48 B) and radiance (16 B) written
+    "raygen": 16,      # per path: ray direction written (bounce 0 reads no other record of a camera ray)
     "reduce": 16,      # per path: radiance read (the image, 12 B per pixel, is added per pixel)
 }
 ADJ_SHADOW_BYTES = 40  # per shadow walk of the adjoint replay: ray (32 B) read, record flag (8 B) rw

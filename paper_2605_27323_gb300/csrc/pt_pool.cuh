@@ -1,4 +1,5 @@
-// pt_pool.cuh -- pooled walks: the dense traversal loop of the wavefront's trace stages.
+// pt_pool.cuh -- pooled walks: the traversal loop of the wavefront's trace stages, of the regenerating megakernel
+// and of the closest-hit queries.
 //
 // A lockstep walk of 32 rays (each lane its own ray, the warp takes 32 new ones when the last has
 // finished) issues every instruction for 9 lanes of 32 on average after the first bounce: lanes whose
@@ -11,11 +12,11 @@
 // and not once per kind.  Each ray visits the nodes and triangles of the lockstep walk in the same
 // order, so hits are the same bit for bit.
 //
-// What bounds it: node data returns to registers at 128 bytes per clock and SM, so a node step (64 bytes
-// a lane) takes 16 cycles of the L1 data path whether 20 or 32 lanes need it: that path is busy 76% of
-// the time (issue 58%, long-scoreboard stalls for the rest) in the launch of bounce 1 at 1080p on 1.15 M
-// triangles.  Against the lockstep walk: extension rays 15.4 -> 22 lanes per node step, bounce 1 9.5 ->
-// 19.7, 683 -> 585 us.
+// What bounds it, in the launch of bounce 1 at 1080p on 1.15 M triangles: the L1 data path, busy 78% of the time with
+// divergent node requests (issue 61%, long-scoreboard stalls for the rest).  Requests fill it, not bytes: a node as
+// two 256-bit loads beats four of 128 bits by 1%, and reading its 56 used bytes in three loads costs 2% on the
+// terrain.  Against the lockstep walk: 168 -> 114 warp instructions per walk, 9.5 -> 18 lanes per instruction, 683
+// -> 531 us; camera rays 117 -> 91, 15 -> 23, 360 -> 282 us.
 #pragma once
 #include "pt_common.cuh"
 
