@@ -8,7 +8,7 @@
  * and Russian roulette (Sec. 3.1).  It runs the estimator two ways (Sec. 2.2 / 2.3): a megakernel
  * (one thread traces one path to termination) and a wavefront pipeline (ray generation, extend
  * traversal, material-sorted shading, shadow traversal, accumulation) linked by device queues
- * with the two-slot active count of Sec. 3.1.  It also provides a path-replay adjoint (gradients
+ * whose active counts (Sec. 3.1) stay on the device.  It also provides a path-replay adjoint (gradients
  * of an image loss with respect to per-material albedo and emission) and batched rendering of
  * many scenes in one persistent wavefront.
  *
