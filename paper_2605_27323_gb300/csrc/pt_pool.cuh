@@ -188,8 +188,11 @@ constexpr uint32_t kAnySlot = 0x80000000u;
 // its first lane's number; it culls every lane that works on the ray, and is the hit at the end: the closest-hit
 // rule makes it independent of the order of the walk (as in trace_closest_group).  When the slots ran out the
 // launches of a 1080p frame lasted another 70 to 80 us, the length of one walk: 1.601 -> 1.547 ms with this, its
-// adjoint 1.700 -> 1.654 ms.
+// adjoint 1.700 -> 1.654 ms.  It goes in phases too: kDrainSteps node steps, a leaf step, then subtrees change hands.
+// 1, 2, 3, 4 steps: the frame 1.485, 1.484, 1.483, 1.489 ms, four 720p frames 2.091, 2.053, 2.037, 2.044 (1.494 and
+// 2.111 with a node or leaf step of each lane in turn).  6, 12 or 20 idle lanes before it starts measure the same.
 constexpr uint32_t kDrainLanes = 12;
+constexpr int kDrainSteps = 3;
 struct DrainShared {
     unsigned long long key[32];       // t | original id of the ray's best hit
     uint32_t tri[32];                 // its triangle (any-hit rays: the caller's `best`)
@@ -226,9 +229,19 @@ __device__ __noinline__ void pool_drain(const Io& io, DrainShared& sh, uint32_t 
         bool hit = false;
         unsigned long long cand = 0ull;
         uint32_t cand_tri = 0u;
-        if (k.ref != kDone) {
-            k.tbest = __uint_as_float((uint32_t)(sh.key[r] >> 32));
-            bool next = false;
+        const auto pop = [&] {
+            k.ref = kDone;
+            while (k.sp > bot) {
+                const uint2 v = stk[--k.sp];
+                if (__uint_as_float(v.y) <= k.tbest * 1.0000005f) {
+                    k.ref = v.x;
+                    break;
+                }
+            }
+        };
+        if (k.ref != kDone) k.tbest = __uint_as_float((uint32_t)(sh.key[r] >> 32));
+#pragma unroll 1
+        for (int rep = 0; rep < kDrainSteps; ++rep) {
             if (!(k.ref & kLeafBit)) {
                 float4 n0, n1, n2;
                 uint2 c;
@@ -239,41 +252,33 @@ __device__ __noinline__ void pool_drain(const Io& io, DrainShared& sh, uint32_t 
                 const bool first0 = h0 && (t0 <= t1 || !h1);
                 k.ref = first0 ? c.x : c.y;
                 if (h0 && h1) stk[k.sp++] = make_uint2(first0 ? c.y : c.x, __float_as_uint(first0 ? t1 : t0));
-                next = !(h0 || h1);
-            } else {
-                const uint32_t first = (k.ref & 0x7FFFFFFFu) >> 3, n_leaf = (k.ref & 7u) + 1u;
-                cand = sh.key[r];
-                for (uint32_t i = 0; i < n_leaf; ++i) {
-                    float t;
-                    uint32_t prim;
-                    if (!tri_test(k.tris, first + i, k.o, k.d, t, prim) || !(t > 0.0f)) continue;
-                    if (rec & kAnyRec) {
-                        hit = hit || t < k.tbest;
-                    } else {
-                        const unsigned long long v = (unsigned long long)__float_as_uint(t) << 32 | prim;
-                        if (v < cand) {
-                            cand = v;
-                            cand_tri = first + i;
-                            hit = true;
-                        }
-                    }
-                }
-                if (hit && !(rec & kAnyRec)) {
-                    atomicMin(&sh.key[r], cand);
-                    k.tbest = __uint_as_float((uint32_t)(cand >> 32));
-                }
-                next = true;
+                else if (!(h0 || h1)) pop();
             }
-            if (next) {
-                k.ref = kDone;
-                while (k.sp > bot) {
-                    const uint2 v = stk[--k.sp];
-                    if (__uint_as_float(v.y) <= k.tbest * 1.0000005f) {
-                        k.ref = v.x;
-                        break;
+            __syncwarp();
+        }
+        if (k.ref != kDone && (k.ref & kLeafBit)) {
+            const uint32_t first = (k.ref & 0x7FFFFFFFu) >> 3, n_leaf = (k.ref & 7u) + 1u;
+            cand = sh.key[r];
+            for (uint32_t i = 0; i < n_leaf; ++i) {
+                float t;
+                uint32_t prim;
+                if (!tri_test(k.tris, first + i, k.o, k.d, t, prim) || !(t > 0.0f)) continue;
+                if (rec & kAnyRec) {
+                    hit = hit || t < k.tbest;
+                } else {
+                    const unsigned long long v = (unsigned long long)__float_as_uint(t) << 32 | prim;
+                    if (v < cand) {
+                        cand = v;
+                        cand_tri = first + i;
+                        hit = true;
                     }
                 }
             }
+            if (hit && !(rec & kAnyRec)) {
+                atomicMin(&sh.key[r], cand);
+                k.tbest = __uint_as_float((uint32_t)(cand >> 32));
+            }
+            pop();
         }
         __syncwarp();
         if (hit && !(rec & kAnyRec) && sh.key[r] == cand) sh.tri[r] = cand_tri;
