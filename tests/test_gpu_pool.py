@@ -128,3 +128,14 @@ def test_pooled_queries(views, large, scene, n):
         t1, p1 = _query(g, few.data_ptr(), m)
         assert torch.equal(t[i:i + m], t1) and torch.equal(prim[i:i + m], p1), i
     assert bool(((prim >= 0) == torch.isfinite(t)).all())
+
+
+# the wavefront's records are added up four floats a load, the megakernel's as three floats
+@pytest.mark.parametrize("spp", [1, 2, 3, 4, 5, 7, 8, 16, 17])
+def test_samples_add_up_alike(views, spp):
+    import torch
+    g, cam = views["soup"]
+    cam = dict(cam, width=37, height=23)
+    a = g.render(cam, spp, 3, 4, mode="wavefront")
+    b = g.render(cam, spp, 3, 4, mode="megakernel")
+    assert torch.equal(a, b)
