@@ -149,12 +149,9 @@ __global__ void __launch_bounds__(128, 8) k_megakernel_pool(DevScene s, DevCamer
             }
             steps = 0;
         }
-        k.node_phase(s, stk);
+        k.node_phase(s, stk, steps);
         k.leaf_phase(s, stk, kind == kWalkShadow);
-        if (++steps >= kMaxSteps) {
-            if (k.ref != kDone) atomicOr(s.status, ST_TRAVERSAL);
-            k.ref = kDone;
-        }
+        k.guard(s, steps);
     }
     warp_add_u64(rays, n_ext);
     warp_add_u64(rays + 1, n_shd);
