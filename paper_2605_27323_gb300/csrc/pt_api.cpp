@@ -721,8 +721,9 @@ pt_status batch_render(pt_scene* const* scenes, const pt_camera* cams, const uin
     };
     const bool use_graph = !(o.flags & PT_FLAG_NO_GRAPH);
     if (use_graph) {
-        // the captured loop depends only on these; tables and counters are read from device memory
-        std::vector<uint64_t> key = {cap, max_depth, n_keys, sort_mode, block, o.rr_start, (uint64_t)fused,
+        // the captured loop depends only on these (all of RenderParams that its kernels read among them); tables
+        // and counters are read from device memory
+        std::vector<uint64_t> key = {cap, max_depth, n_keys, sort_mode, block, o.rr_start, (uint64_t)fused, p.mis,
                                      (uint64_t)__builtin_bit_cast(uint32_t, o.rr_fixed),
                                      (uint64_t)(uintptr_t)ctx->tables.p, (uint64_t)(uintptr_t)ctx->wf.p, n};
         if (!ctx->graph || ctx->graph_key != key) {
