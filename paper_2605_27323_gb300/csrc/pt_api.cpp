@@ -651,11 +651,12 @@ pt_status batch_render(pt_scene* const* scenes, const pt_camera* cams, const uin
         waves.push_back(wv);
     }
     std::vector<char> blob;
-    const size_t o_sc = put(blob, views.data(), n), o_cam = put(blob, dcs.data(), n), o_off = put(blob, off.data(), n + 1),
-                 o_spp = put(blob, spps.data(), n), o_out = put(blob, outs.data(), n),
-                 o_px = put(blob, px_off.data(), n + 1), o_seg = put(blob, segs.data(), segs.size());
+    // the captured bounce loop reads the tables up to the seed by address: their places depend on n alone.  The wave
+    // segments, whose number depends on the views, come last.
     const unsigned long long seed64 = seed;
-    const size_t o_seed = put(blob, &seed64, 1);
+    const size_t o_sc = put(blob, views.data(), n), o_cam = put(blob, dcs.data(), n), o_off = put(blob, off.data(), n + 1),
+                 o_spp = put(blob, spps.data(), n), o_out = put(blob, outs.data(), n), o_seed = put(blob, &seed64, 1),
+                 o_px = put(blob, px_off.data(), n + 1), o_seg = put(blob, segs.data(), segs.size());
     if (ctx->tables.bytes < blob.size() && ctx->graph) {
         cudaGraphExecDestroy(ctx->graph);
         ctx->graph = nullptr;

@@ -31,3 +31,17 @@ def test_batches_of_one_shape_with_and_without_mis(scene, order):
         for o, c, spp in zip(outs, cams, [2, 4]):
             assert torch.equal(o, g.render(c, spp, 5, 7, mis=mis)), mis
     assert not torch.equal(g.render(cams[1], 4, 5, 7, mis=False), g.render(cams[1], 4, 5, 7, mis=True))
+
+
+# the waves of the first view hold one segment, those of the others 4, 16 and 64 (32 bytes each): the tables that
+# follow the segments move
+@pytest.mark.parametrize("sizes", [(8, 16, 32, 64), (64, 32, 16, 8)])
+def test_batches_of_one_shape_with_other_image_sizes(scene, sizes):
+    import torch
+
+    import paper_2605_27323_gb300 as pt
+    g, cam = scene
+    for k, size in enumerate(sizes):
+        c = dict(cam, width=size, height=size)
+        out, = pt.render_batch([g], [c], [1], 5, 100 + k, queue_capacity=64)
+        assert torch.equal(out, g.render(c, 1, 5, 100 + k)), size
