@@ -206,6 +206,13 @@ struct pt_scene {
         return PT_OK;
     }
 
+    // For a call that fails before its ray generation, which clears the counters: it has traced nothing, and
+    // pt_get_stats must not find the counts of the call before it.
+    pt_status failed(pt_status s, cudaStream_t st) {
+        if (cudaMemsetAsync(counters.p, 0, counters.bytes, st) != cudaSuccess) cudaGetLastError();
+        return s;
+    }
+
     void ev_reset(bool on) {
         profiling = on;
         ev_used = 0;
@@ -391,7 +398,7 @@ pt_status run_wavefront(pt_scene* sc, const pt::DevCamera& cam, const pt::Render
     uint64_t cap = o.queue_capacity ? std::min<uint64_t>(o.queue_capacity, n_paths) : n_paths;
     cap = std::max<uint64_t>(cap - cap % p0.spp, p0.spp);
     if (cap >= (1ull << 32)) cap = ((1ull << 32) - (1ull << 20)) / p0.spp * p0.spp;
-    PT_TRY(sc->ensure_wf(cap));
+    if (pt_status s = sc->ensure_wf(cap); s != PT_OK) return sc->failed(s, st);
     pt::WfBuffers w = sc->wfb;
     pt::carve_counters(sc->counters.p, w);
     w.sig = sig;
@@ -1399,9 +1406,10 @@ pt_status pt_render_backward(pt_scene* sc, const pt_camera* cam, uint32_t spp, u
         uint64_t cap = std::min<uint64_t>(n_paths, (8ull << 30) / per_path);
         cap = std::max<uint64_t>(cap - cap % spp, spp);
         if (cap >= (1ull << 32)) cap = ((1ull << 32) - (1ull << 20)) / spp * spp;
-        PT_TRY(sc->ensure_wf(cap));
         const size_t rec_bytes = align256(cap * max_depth * 64);
-        PT_TRY(sc->adj.ensure(rec_bytes + align256(cap * 4)));
+        pt_status room = sc->ensure_wf(cap);
+        if (room == PT_OK) room = sc->adj.ensure(rec_bytes + align256(cap * 4));
+        if (room != PT_OK) return sc->failed(room, st);
         pt::WfBuffers w = sc->wfb;
         pt::carve_counters(sc->counters.p, w);
         w.sig = nullptr;
