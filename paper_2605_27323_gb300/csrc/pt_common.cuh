@@ -180,7 +180,9 @@ __device__ __forceinline__ float3 mk_path(const DevScene& s, const DevCamera& c,
     float prev_pdf = 0.f;
     for (uint32_t b = 0; b < p.max_depth; ++b) {
         ++n_ext;
-        Hit h = trace_closest<INST, 0, !INST>(s, o, d);        // step 2
+        Hit h;                                                 // step 2
+        if constexpr (INST) h = trace_closest_inst<false, false>(s, o, d);
+        else h = trace_closest(s, o, d);
         if (h.tri == kMiss) {
             L = add_rn(L, mul_rn(tp, env));
             rec.ev(b, 0, kMiss, __int_as_float(0x7f800000), tp.x);
@@ -194,7 +196,10 @@ __device__ __forceinline__ float3 mk_path(const DevScene& s, const DevCamera& c,
             uint32_t vis = 0;
             if (V.cast) {
                 ++n_shd;
-                vis = trace_any<INST, 0, !INST>(s, V.s_o, V.s_d, V.s_tmax) ? 0u : 1u;
+                bool occluded;
+                if constexpr (INST) occluded = trace_any_inst<false, false>(s, V.s_o, V.s_d, V.s_tmax);
+                else occluded = trace_any(s, V.s_o, V.s_d, V.s_tmax);
+                vis = occluded ? 0u : 1u;
                 if (vis) L = add_rn(L, V.contrib);
             }
             rec.ev(b, 1, (V.light_j << 2) | ((uint32_t)V.cast << 1) | vis, V.nee_cx, V.nee_cl);

@@ -127,10 +127,21 @@ __device__ __forceinline__ bool tri_test(const float4* __restrict__ tris, uint32
 }
 
 // One node: two 256-bit loads (node records are 64-byte aligned; 2.055 -> 2.046 ms per 1080p frame against four of 128
-// bits).
+// bits).  WIDE = false: four of 128 bits, which are the faster ones in the two-level walks of the megakernel in the
+// paper's layout (the 1080p frame of 200 placed spheres 14.46 -> 13.80 ms, at the same registers and spills); the
+// single-level walks, the adjoint's and the hybrid's measure the same either way.
+template <bool WIDE = true>
 __device__ __forceinline__ void load_node(const float4* __restrict__ nodes, uint32_t i, float4& n0, float4& n1,
                                           float4& n2, uint2& refs) {
     const float4* p = nodes + 4 * (size_t)i;
+    if constexpr (!WIDE) {
+        n0 = __ldg(p);
+        n1 = __ldg(p + 1);
+        n2 = __ldg(p + 2);
+        const float4 n3 = __ldg(p + 3);
+        refs = make_uint2(__float_as_uint(n3.x), __float_as_uint(n3.y));
+        return;
+    }
     [[maybe_unused]] float pad0, pad1;
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(n0.x), "=f"(n0.y), "=f"(n0.z), "=f"(n0.w), "=f"(n1.x), "=f"(n1.y), "=f"(n1.z), "=f"(n1.w)
@@ -576,7 +587,7 @@ __device__ __forceinline__ InstRay instance_ray(const DevScene& s, uint32_t k, f
 }
 
 // Closest hit inside one mesh (object-space ray), updating the running best over instances.
-template <bool PK = true>
+template <bool PK = true, bool WIDE = true>
 __device__ __forceinline__ void blas_closest(const DevScene& s, const InstRay& r, uint32_t k, float& tbest,
                                              uint32_t& best, uint32_t& bprim, uint32_t& binst, uint32_t& steps) {
     const float3 id = ray_rcp(r.d);
@@ -588,7 +599,7 @@ __device__ __forceinline__ void blas_closest(const DevScene& s, const InstRay& r
         if (!(ref & kLeafBit)) {
             float4 n0, n1, n2;
             uint2 c;
-            load_node(s.nodes, ref, n0, n1, n2, c);
+            load_node<WIDE>(s.nodes, ref, n0, n1, n2, c);
             float t0, t1;
             bool h0, h1;
             box_test2<PK>(n0, n1, n2, r.o, id, tbest, t0, t1, h0, h1);
@@ -641,7 +652,7 @@ __device__ __forceinline__ void blas_closest(const DevScene& s, const InstRay& r
     }
 }
 
-template <bool PK = true>
+template <bool PK = true, bool WIDE = true>
 __device__ __forceinline__ bool blas_any(const DevScene& s, const InstRay& r, float tmax, uint32_t& steps) {
     const float3 id = ray_rcp(r.d);
     uint32_t stack_ref[kStack];
@@ -651,7 +662,7 @@ __device__ __forceinline__ bool blas_any(const DevScene& s, const InstRay& r, fl
         if (!(ref & kLeafBit)) {
             float4 n0, n1, n2;
             uint2 c;
-            load_node(s.nodes, ref, n0, n1, n2, c);
+            load_node<WIDE>(s.nodes, ref, n0, n1, n2, c);
             float t0, t1;
             bool h0, h1;
             box_test2<PK>(n0, n1, n2, r.o, id, tmax, t0, t1, h0, h1);
@@ -683,7 +694,7 @@ __device__ __forceinline__ bool blas_any(const DevScene& s, const InstRay& r, fl
     }
 }
 
-template <bool PK = true>
+template <bool PK = true, bool WIDE = true>
 __device__ __forceinline__ Hit trace_closest_inst(const DevScene& s, float3 o, float3 d) {
     const float3 id = ray_rcp(d);
     float tbest = __int_as_float(0x7f800000);
@@ -697,7 +708,7 @@ __device__ __forceinline__ Hit trace_closest_inst(const DevScene& s, float3 o, f
         if (!(ref & kLeafBit)) {
             float4 n0, n1, n2;
             uint2 c;
-            load_node(s.tlas, ref, n0, n1, n2, c);
+            load_node<WIDE>(s.tlas, ref, n0, n1, n2, c);
             float t0, t1;
             bool h0, h1;
             box_test2<PK>(n0, n1, n2, o, id, tbest, t0, t1, h0, h1);
@@ -720,7 +731,7 @@ __device__ __forceinline__ Hit trace_closest_inst(const DevScene& s, float3 o, f
             uint32_t first = (ref & 0x7FFFFFFFu) >> 3, cnt = (ref & 7u) + 1u;
             for (uint32_t q = 0; q < cnt; ++q) {
                 const InstRay r = instance_ray(s, first + q, o, d);
-                blas_closest<PK>(s, r, first + q, tbest, best, bprim, binst, steps);
+                blas_closest<PK, WIDE>(s, r, first + q, tbest, best, bprim, binst, steps);
             }
         }
         if (steps >= kMaxSteps) {
@@ -747,7 +758,7 @@ __device__ __forceinline__ Hit trace_closest_inst(const DevScene& s, float3 o, f
     return h;
 }
 
-template <bool PK = true>
+template <bool PK = true, bool WIDE = true>
 __device__ __forceinline__ bool trace_any_inst(const DevScene& s, float3 o, float3 d, float tmax) {
     const float3 id = ray_rcp(d);
     uint32_t stack_ref[kStack];
@@ -758,7 +769,7 @@ __device__ __forceinline__ bool trace_any_inst(const DevScene& s, float3 o, floa
         if (!(ref & kLeafBit)) {
             float4 n0, n1, n2;
             uint2 c;
-            load_node(s.tlas, ref, n0, n1, n2, c);
+            load_node<WIDE>(s.tlas, ref, n0, n1, n2, c);
             float t0, t1;
             bool h0, h1;
             box_test2<PK>(n0, n1, n2, o, id, tmax, t0, t1, h0, h1);
@@ -775,7 +786,7 @@ __device__ __forceinline__ bool trace_any_inst(const DevScene& s, float3 o, floa
         } else {
             uint32_t first = (ref & 0x7FFFFFFFu) >> 3, cnt = (ref & 7u) + 1u;
             for (uint32_t q = 0; q < cnt; ++q)
-                if (blas_any<PK>(s, instance_ray(s, first + q, o, d), tmax, steps)) return true;
+                if (blas_any<PK, WIDE>(s, instance_ray(s, first + q, o, d), tmax, steps)) return true;
         }
         if (steps >= kMaxSteps) {
             atomicOr(s.status, ST_TRAVERSAL);
