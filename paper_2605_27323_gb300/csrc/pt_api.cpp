@@ -192,6 +192,8 @@ struct pt_scene {
     // 2.187 -> 2.148; the 36-triangle box, whose walks are over in a few steps, 249 -> 270 us.
     static constexpr uint64_t kShareNodes = 1u << 14;
     uint32_t shares_walks() const { return !instanced && n_nodes >= kShareNodes ? 1u : 0u; }
+    // Trees of a few nodes, whose walks are over in a handful of steps.
+    bool small_tree() const { return n_nodes < 64; }
     uint32_t* status() const { return counters.as<uint32_t>() + pt::kStatusWord; }
     pt_status ensure_counters() { return counters.ensure(pt::kCounterBytes); }
     unsigned long long* trav() const { return hist() + 132; }   // 4 traversal counters
@@ -1480,8 +1482,19 @@ pt_status pt_trace_closest(pt_scene* sc, const float* d_rays, uint32_t n, float*
     PT_TRY(set_device(sc));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     sc->last_stream = st;
-    PT_CUDA(pt::launch_trace_closest(launch_for(sc, pt::K_EXTEND, 0, 256, st, n), sc->view(), d_rays, n, d_t, d_prim,
-                                     sc->shares_walks() != 0u));
+    // a warp's rays are dealt in runs of 32 here, so more blocks than runs would only stand idle
+    pt::Launch l = launch_for(sc, pt::K_EXTEND, 0, 256, st, n);
+    l.grid = (int)std::min<uint64_t>((uint64_t)l.grid, ((uint64_t)n + 255) / 256);
+    // In the queries below the pool has nothing to hand out, and its votes only lengthen each walk's chain of node loads.
+    // A few rays: one ray on 3.9 k nodes 16.8 us pooled, 12.8 us one ray per thread, 6 rays 20.8 and 16.9, on two levels
+    // of 33 nodes 8.4 and 6.6; with 12 the two measure alike, from 24 on pools are ahead on all but the smallest trees.
+    // With shared ends 8 rays gain on 22 k nodes (21.8 pooled, 26.9) and measure alike on 610 k (28.9, 29.0), 4 do not
+    // (18.7, 18.8 and 20.9, 18.9).  One ray a thread on a tree of a few nodes: 10,000 rays on 19 nodes 12.6 pooled,
+    // 10.8; on 39 and 95 nodes alike; on 922 29.0 pooled, 33.2; on two levels of 33 nodes pools are ahead.
+    const bool shares = sc->shares_walks() != 0u;
+    const bool lockstep = n <= (shares ? 4u : 8u) ||
+                          (sc->small_tree() && !sc->instanced && (uint64_t)l.grid * l.block >= n);
+    PT_CUDA(pt::launch_trace_closest(l, sc->view(), d_rays, n, d_t, d_prim, shares, lockstep));
     return PT_OK;
 }
 

@@ -50,6 +50,20 @@ __global__ void __launch_bounds__(256, INST ? 4 : 5) k_trace_closest(const __gri
     pool_walk<INST, SHARE>(s, q, n, QueryIo<INST>{s, rays, t, prim});
 }
 
+// The same, each thread one ray at a time.
+template <bool INST>
+__global__ void __launch_bounds__(256) k_trace_closest_lockstep(DevScene s, const float* __restrict__ rays, uint32_t n,
+                                                                float* __restrict__ t, int32_t* __restrict__ prim) {
+    const uint32_t stride = gridDim.x * blockDim.x;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const float* r = rays + 8 * (size_t)i;
+        const Hit h = trace_closest<INST>(s, f3(__ldg(r), __ldg(r + 1), __ldg(r + 2)),
+                                          f3(__ldg(r + 4), __ldg(r + 5), __ldg(r + 6)));
+        t[i] = h.t;
+        prim[i] = h.tri == kMiss ? -1 : (int32_t)h.prim;
+    }
+}
+
 __global__ void k_debug_rng(uint64_t seed, const uint32_t* px, const uint32_t* sm, const uint32_t* bo,
                             const uint32_t* dm, uint32_t n, float* out) {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -65,7 +79,12 @@ cudaError_t launch_set_materials(cudaStream_t st, DevMat* mats, uint32_t n, cons
 }
 
 cudaError_t launch_trace_closest(const Launch& l, const DevScene& s, const float* rays, uint32_t n, float* t,
-                                 int32_t* prim, bool share) {
+                                 int32_t* prim, bool share, bool lockstep) {
+    if (lockstep) {
+        if (s.tlas) k_trace_closest_lockstep<true><<<l.grid, l.block, 0, l.st>>>(s, rays, n, t, prim);
+        else k_trace_closest_lockstep<false><<<l.grid, l.block, 0, l.st>>>(s, rays, n, t, prim);
+        return cudaGetLastError();
+    }
     // a slot of the pool has 31 bits
     for (uint64_t i = 0; i < n; i += 1u << 30) {
         const uint32_t m = (uint32_t)std::min<uint64_t>(n - i, 1u << 30);

@@ -98,9 +98,9 @@ cudaError_t launch_adjoint_reverse(const Launch& l, const DevScene& s, const Ren
 
 // Utilities.
 cudaError_t launch_set_materials(cudaStream_t st, DevMat* mats, uint32_t n, const float* albedo, const float* emission);
-// share: the tree is large enough for shared last walks (pool_drain)
+// share: the tree is large enough for shared last walks (pool_drain); lockstep: one ray per thread instead of pooled walks
 cudaError_t launch_trace_closest(const Launch& l, const DevScene& s, const float* rays, uint32_t n, float* t,
-                                 int32_t* prim, bool share);
+                                 int32_t* prim, bool share, bool lockstep);
 cudaError_t launch_debug_rng(const Launch& l, uint64_t seed, const uint32_t* px, const uint32_t* sm,
                              const uint32_t* bo, const uint32_t* dm, uint32_t n, float* out);
 
