@@ -855,8 +855,14 @@ pt_status render_impl(pt_scene* sc, const pt_camera* cam, uint32_t spp, uint32_t
                                                         : short_stack_kernel(sc, pt::K_MEGA_REGEN, p.short_stack),
                                       o.block_size ? std::min<uint32_t>(o.block_size, 128) : 128, 128,
                                       st, n_paths);
+            // A tree of a few nodes and hardly more paths than threads: walks are over in a handful of steps and most of
+            // the work is shading, which the pooled form keeps waiting until 20 lanes have ended.  The 14-node box at
+            // 128 x 128 x 16, depth 8: 261 us pooled, 248 in lockstep; 61 x 47, depth 8: 122 and 101; 19 nodes, two
+            // levels of 33 nodes at 128 x 128 x 16: 111 and 101, 178 and 167.  From two paths a thread on the pooled
+            // form is ahead (the box at 512 x 256 x 4: 243 and 260 us), on 95 nodes at any size (148 and 170).
+            const bool lockstep = sc->small_tree() && n_paths <= 2ull * (uint64_t)l.grid * (uint64_t)l.block;
             PT_CUDA(pt::launch_megakernel_regen(l, sc->view(), dc, p, n_paths, outL, img, o.d_path_sig, sc->rays(),
-                                                sc->next_path()));
+                                                sc->next_path(), lockstep));
         }
         PT_TRY(sc->ev_end(ev, st));
         sc->launches += 1;

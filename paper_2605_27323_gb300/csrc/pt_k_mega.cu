@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(128, 8) k_megakernel_pool(DevScene s, DevCamer
     warp_add_u64(rays + 1, n_shd);
 }
 
-// Lockstep form of the short-stack and counting variants: one bounce per loop iteration.
+// Lockstep form: one bounce per loop iteration (the short-stack and counting variants, small renders of tiny trees).
 // Register cap for 8 resident blocks of 128: occupancy outweighs the spills (measured 3.96 -> 3.11 ms
 // per 1080p frame against the uncapped 107 registers).
 template <bool SIG, bool MIS, bool INST, int SK = 0, bool CNT = false>
@@ -315,11 +315,15 @@ __global__ void k_finish_commit(WfBuffers w, uint32_t b0, uint32_t threshold, un
 // ------------------------------------------------------------------ launchers
 cudaError_t launch_megakernel_regen(const Launch& l, const DevScene& s, const DevCamera& c, const RenderParams& p,
                                     uint64_t n_paths, float* out_L, float* img, uint32_t* sig, unsigned long long* rays,
-                                    unsigned long long* next_path) {
+                                    unsigned long long* next_path, bool lockstep) {
     // PT_FLAG_SHORT_STACK: the single-level variants keep their top stack entries in shared memory
     const size_t sm = stack_smem_bytes(kShortStack, l.block);
 #define PT_REGEN(S, M, I, K) k_megakernel_regen<S, M, I, K><<<l.grid, l.block, K ? sm : 0, l.st>>>(s, c, p, n_paths, out_L, img, sig, rays, next_path)
-#define PT_POOL(S, M, I) k_megakernel_pool<S, M, I><<<l.grid, l.block, 0, l.st>>>(s, c, p, n_paths, out_L, img, sig, rays, next_path)
+#define PT_POOL(S, M, I)                       \
+    do {                                       \
+        if (lockstep) PT_REGEN(S, M, I, 0);    \
+        else k_megakernel_pool<S, M, I><<<l.grid, l.block, 0, l.st>>>(s, c, p, n_paths, out_L, img, sig, rays, next_path); \
+    } while (0)
     if (s.tlas) {            // two-level scenes: one variant, MIS decided at run time
         if (sig) PT_POOL(true, true, true);
         else PT_POOL(false, true, true);

@@ -21,10 +21,11 @@ cudaError_t launch_megakernel(const Launch& l, const DevScene& s, const DevCamer
                               uint64_t n_paths, float* out_L, float* img, uint32_t* sig,
                               unsigned long long* rays);
 
-// Persistent megakernel with path regeneration (next_path: device counter zeroed by the caller).
+// Persistent megakernel with path regeneration (next_path: device counter zeroed by the caller).  lockstep: one bounce
+// per loop iteration instead of pooled walks.
 cudaError_t launch_megakernel_regen(const Launch& l, const DevScene& s, const DevCamera& c, const RenderParams& p,
                                     uint64_t n_paths, float* out_L, float* img, uint32_t* sig, unsigned long long* rays,
-                                    unsigned long long* next_path);
+                                    unsigned long long* next_path, bool lockstep);
 
 // Event logs of selected paths (testing aid).
 cudaError_t launch_debug_paths(cudaStream_t st, const DevScene& s, const DevCamera& c, const RenderParams& p,
