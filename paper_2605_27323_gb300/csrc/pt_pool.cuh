@@ -35,9 +35,10 @@ constexpr uint32_t kIdleLanes = 20;
 // and a leaf phase -- a walk that stands above the depth is given up, and so are all walks of a warp that has counted
 // kMaxWarpSteps since its lanes last took slots.  A turn takes every walking lane a step on and a repeated node step at
 // least kNodeLanes of them, so walks of up to kMaxSteps steps never meet that count.  A look at the stack at every push
-// instead costs 2% of the 1080p frame and 3% of its two-level form, a count at every node step 1%; counting every other
-// step, with the stack looked at once a turn: the frame 1.485 -> 1.490 ms, its two-level form 1.580 -> 1.597, the
-// megakernel's 1.900 -> 1.922, the terrain 9.49 -> 9.53.
+// instead costs 2% of the 1080p frame and 3% of its two-level form, a count at every node step 1%.  With the stack looked
+// at once a turn and every other step counted: the frame 1.485 -> 1.490 ms, the megakernel's 1.900 -> 1.922, the terrain
+// 9.49 -> 9.53.  Two levels count every step, where a second copy of the step costs more than the count: the frame
+// 1.580 -> 1.594 ms (1.597 by twos), the megakernel's 2.217 -> 2.261 (2.334).
 constexpr uint32_t kPhaseSteps = 64;
 constexpr uint32_t kMaxWarpSteps = (32u / kNodeLanes + 1u) * kMaxSteps;
 
@@ -128,7 +129,7 @@ struct Walker {
             }
         }
     }
-    // Node steps while at least kNodeLanes lanes hold an inner node, kPhaseSteps at most; counted in `steps` by twos.
+    // Node steps while at least kNodeLanes lanes hold an inner node, kPhaseSteps at most; counted in `steps`.
     __device__ __forceinline__ void node_phase(const DevScene& s, Stack& stk, uint32_t& steps) {
         const auto step = [&]() -> bool {
             if (!(ref & kLeafBit)) {
@@ -146,10 +147,16 @@ struct Walker {
             }
             return (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, !(ref & kLeafBit))) >= kNodeLanes;
         };
-        uint32_t pairs = 0;
-        while (step() && step() && ++pairs < kPhaseSteps / 2u) {
+        uint32_t i = 0;
+        if constexpr (INST) {
+            while (step() && ++i < kPhaseSteps) {
+            }
+            steps += i;
+        } else {
+            while (step() && step() && ++i < kPhaseSteps / 2u) {
+            }
+            steps += 2u * i;
         }
-        steps += 2u * pairs;
     }
     // One leaf step of the lanes that hold a leaf; `any`: the lane's walk is an any-hit one.
     __device__ __forceinline__ void leaf_phase(const DevScene& s, Stack& stk, bool any) {
