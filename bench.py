@@ -52,18 +52,35 @@ BYTES_PER_UNIT = {
     "shadow": 80,      # per shadow ray: o|tmax + d|id (32 B) + contribution (16 B) read, L rw (32 B)
     "shade": 184,      # per active path: ray+tp (48) + hit (8) + L rw (32) + next ray (48) + shadow (48)
     "megakernel": 12,  # per path: radiance written (scene reads amortise to ~0 per path)
-    "raygen": 16,      # per path: ray direction written (bounce 0 reads no other record of a camera ray)
+    "raygen": 16,      # per path: ray direction written
     "reduce": 16,      # per path: radiance read (the image, 12 B per pixel, is added per pixel)
 }
+# The same at bounce 0: of a camera ray only the direction is stored, its origin (16 B, read by extend and by shade),
+# throughput (16 B) and radiance (16 B) are known.
+CAMERA_BYTES_PER_UNIT = {"extend": 24, "shade": 136}
 ADJ_SHADOW_BYTES = 40  # per shadow walk of the adjoint replay: ray (32 B) read, record flag (8 B) rw
 
 
 def wavefront_frame_bytes(st: dict, n_paths: int, n_pixels: int) -> float:
-    """Algorithmic bytes of one wavefront frame from its device counts: every stage's per-unit
-    bytes times the units it processed (extension rays = paths entering each bounce)."""
+    """Bytes of one wavefront frame from its device counts if every path's records came from the
+    queues: every stage's per-unit bytes times the units it processed (extension rays = paths entering
+    each bounce)."""
     ext = float(sum(st["active"]))
     return (ext * (BYTES_PER_UNIT["extend"] + BYTES_PER_UNIT["shade"]) + st["shadow_rays"] * BYTES_PER_UNIT["shadow"]
             + n_paths * (BYTES_PER_UNIT["raygen"] + BYTES_PER_UNIT["reduce"]) + n_pixels * 12)
+
+
+def frame_bytes(st: dict, n_paths: int, n_pixels: int) -> float:
+    """Algorithmic bytes of one wavefront frame: wavefront_frame_bytes without what bounce 0 does not read."""
+    spared = sum(BYTES_PER_UNIT[k] - CAMERA_BYTES_PER_UNIT[k] for k in CAMERA_BYTES_PER_UNIT)
+    return wavefront_frame_bytes(st, n_paths, n_pixels) - spared * float(st["active"][0] if st["active"] else 0)
+
+
+def extend_stage_bytes(ext: float, camera: float, shadow_fwd: float, shadow_adj: float) -> float:
+    """Algorithmic bytes of extend-stage launches that walk `ext` extension rays, `camera` of them camera rays, and
+    the shadow rays of forward frames and of adjoint replays."""
+    return (BYTES_PER_UNIT["extend"] * (ext - camera) + CAMERA_BYTES_PER_UNIT["extend"] * camera
+            + BYTES_PER_UNIT["shadow"] * shadow_fwd + ADJ_SHADOW_BYTES * shadow_adj)
 
 
 def traversal_ceilings(units_per_launch: float, avg_launch_ms: float, nodes_per_unit: float, tris_per_unit: float,
@@ -380,7 +397,7 @@ def run_gpu(args):
     # The roofline is reported for the wavefront's extend-stage launches (forward + adjoint replay):
     # k_extend at bounce 0 and k_trace after it, which in the default fused order also walks the
     # shadow rays of the previous bounce.  Their algorithmic bytes are the queue records they move:
-    # 40 B per extension walk and 80 B per shadow walk; the unit is one walk.  The megakernel, whose
+    # 40 B per extension walk (24 of a camera ray) and 80 B per shadow walk; the unit is one walk.  The megakernel, whose
     # total time is similar, keeps each path's state in registers (12 B of radiance written per path),
     # so an HBM roofline does not bound it; every kernel's share of the step is listed beside the
     # roofline, and the traversal ceilings of both kernels next to it.
@@ -390,8 +407,8 @@ def run_gpu(args):
     shd_adj = sum(r[5]["shadow_rays"] for r in recs)
     walks = units["extend"] + ((shd_fwd + shd_adj) if fused else 0)
     # an adjoint shadow walk reads its ray (32 B) and sets the record's visibility flag (8 B)
-    alg_bytes = (BYTES_PER_UNIT["extend"] * units["extend"]
-                 + ((BYTES_PER_UNIT["shadow"] * shd_fwd + ADJ_SHADOW_BYTES * shd_adj) if fused else 0))
+    alg_bytes = extend_stage_bytes(units["extend"], 2 * sum(r[3]["active"][0] for r in recs), shd_fwd if fused else 0,
+                                   shd_adj if fused else 0)
     kernel_ms = {k: stage[k] for k in ("extend", "shadow", "shade", "megakernel", "sort", "raygen", "reduce")}
     kernel_ms["adjoint_other"] = max(0.0, stage["adjoint_total"] - sum(r[5][k] for r in recs for k in
                                                                      ("ms_extend", "ms_shade", "ms_shadow",
@@ -414,7 +431,7 @@ def run_gpu(args):
 
     wf_frame = float(np.mean(wf_ms))
     mk_frame = float(np.mean(mk_ms))
-    wf_bytes = float(np.mean([wavefront_frame_bytes(r[3], n_paths, W * H) for r in recs]))
+    wf_bytes = float(np.mean([frame_bytes(r[3], n_paths, W * H) for r in recs]))
     wf_bpr = wf_bytes / float(np.mean(wf_rays))
     wf_roof = {"bound": "hbm", "algorithmic_bytes_per_frame": wf_bytes, "bytes_per_ray": wf_bpr,
                "achieved": wf_bytes / (wf_frame * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
