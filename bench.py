@@ -404,7 +404,8 @@ def run_gpu(args):
     dom = "extend"
     fused = launches["shadow"] == 0
     shd_fwd = sum(r[3]["shadow_rays"] for r in recs)
-    shd_adj = sum(r[5]["shadow_rays"] for r in recs)
+    # the replay of a frame's seed casts the frame's shadow rays again (the library counts rays for renders only)
+    shd_adj = shd_fwd
     walks = units["extend"] + ((shd_fwd + shd_adj) if fused else 0)
     # an adjoint shadow walk reads its ray (32 B) and sets the record's visibility flag (8 B)
     alg_bytes = extend_stage_bytes(units["extend"], 2 * sum(r[3]["active"][0] for r in recs), shd_fwd if fused else 0,
@@ -498,7 +499,9 @@ def run_gpu(args):
         row["hybrid_over_mk"] = row["megakernel_ms"] / row["hybrid_ms"]
         depth_sweep[str(dmax)] = row
     # traversal work per ray (device counters of the counting instantiations; outside the timed region):
-    # the wavefront's extend walks per extension ray, the megakernel's walks per path
+    # the wavefront's extend walks per extension ray, the megakernel's walks per path.  The counting kernels walk one
+    # ray per lane in lockstep: the pooled walks make the same visits, launches with groups of lanes and with shared ends
+    # (the sparse bounces, the last walks of a launch) some more.
     g.render(cam, spp, depth, 0, mode="wavefront", rr_start=3, count_traversal=True)
     cw = g.stats()
     g.render(cam, spp, depth, 0, mode="megakernel", rr_start=3, count_traversal=True)
