@@ -189,7 +189,8 @@ struct pt_scene {
 
     // Large trees: the ends of the fused order's trace launches share walks (pool_drain).  The 1080p frame of 1.15 M
     // triangles (0.6 M nodes) 1.602 -> 1.548 ms, of 0.22 M triangles 1.442 -> 1.429, four 720p frames of 95 k triangles
-    // 2.187 -> 2.148; the 36-triangle box, whose walks are over in a few steps, 249 -> 270 us.
+    // 2.187 -> 2.148; the 36-triangle box, whose walks are over in a few steps, 249 -> 270 us.  Between the box's 14 nodes
+    // and the 48 k of 95 k triangles nothing was measured.
     static constexpr uint64_t kShareNodes = 1u << 14;
     uint32_t shares_walks() const { return !instanced && n_nodes >= kShareNodes ? 1u : 0u; }
     // Trees of a few nodes, whose walks are over in a handful of steps.
@@ -360,7 +361,8 @@ pt::Launch launch_for(const pt_scene* sc, int kernel, uint32_t block_opt, uint32
     uint64_t grid = (uint64_t)sm_count(sc->device) * (uint64_t)per;
     uint64_t need = (work_upper + l.block - 1) / l.block;
     // the walks of a small image: four times the blocks, so that they spread over more SMs, fewer to a warp, and a
-    // sparse bounce's rays get more lanes each (61 x 47 pixels, depth 4: 77.7 -> 66.2 us; 8 and 16 times: 66.7, 68.2)
+    // sparse bounce's rays get more lanes each (61 x 47 pixels, depth 4, the one size swept: 77.7 -> 66.2 us; 8 and 16
+    // times: 66.7, 68.2)
     if (kernel == pt::K_EXTEND || kernel == pt::K_TRACE || kernel == pt::K_EXTEND_INST || kernel == pt::K_TRACE_INST)
         need *= 4;
     if (need < grid) grid = need;

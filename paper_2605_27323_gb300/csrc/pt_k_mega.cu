@@ -21,9 +21,9 @@ constexpr uint32_t kMegaIdleLanes = 20;
 // Pooled form: the lanes' walks, of rays and of shadow rays, are stepped together (Walker).  When kMegaIdleLanes
 // of them have ended -- or as many as are still walking -- those lanes shade, add their shadow ray's
 // contribution or take a new path, and begin their next walk.  One bounce per iteration in lockstep
-// (k_megakernel_regen below) issued for 6.2 of 32 lanes; the 1080p frame 2.99 -> 1.95 ms.  16 and 22 lanes
+// (k_megakernel_regen below) issued for 6.2 of 32 lanes; the 1080p frame 2.99 -> 1.92 ms.  16 and 22 lanes
 // measured the same, 12 2.04 ms (shading, some 700 instructions, runs too often for too few).
-// Registers capped for 8 resident blocks of 128 (64 registers, 306 bytes of spills, nearly all around
+// Registers capped for 8 resident blocks of 128 (64 registers, 318 bytes of spills, nearly all around
 // shading): 6 blocks measured 2.01 ms.
 template <bool SIG, bool MIS, bool INST>
 __global__ void __launch_bounds__(128, 8) k_megakernel_pool(DevScene s, DevCamera c, RenderParams p, uint64_t n_paths,

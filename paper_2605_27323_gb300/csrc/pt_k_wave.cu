@@ -126,9 +126,9 @@ struct TraceIo {
     }
 };
 
-// Resident blocks of 256 of the traversal kernels, which cap their registers.  Pooled walks: 5 (48 registers,
-// no spills; against 6 blocks with 80 bytes of spills 1.94 -> 1.91 ms per 1080p frame, against 4 blocks
-// 1.96 -> 1.91).  Lockstep walks (short stack, counting): 6 single-level (40 registers), 4 two-level (64
+// Resident blocks of 256 of the traversal kernels, which cap their registers.  Pooled walks: 5 (48 registers; no spills
+// in the loop without shared ends, up to 16 bytes with them and 92 in the shared end itself, 44 in the batch's form;
+// against 6 blocks with 80 bytes of spills 1.94 -> 1.91 ms per 1080p frame, against 4 blocks 1.96 -> 1.91).  Lockstep walks (short stack, counting): 6 single-level (40 registers), 4 two-level (64
 // registers; 6 blocks measured slower, and without a bound ptxas takes 78 registers, leaving 3 blocks:
 // 2.89 -> 3.00 ms per two-level frame).
 constexpr int trace_blocks(bool inst, bool pooled) { return inst ? 4 : pooled ? 5 : 6; }
@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(256) k_shadow(Src src, WfBuffers w, uint32_t b
 constexpr uint32_t kCoopMinLanes = 2u;
 // Groups of two lanes only below this many walks: from there on the pooled walk is the faster one (the launch of
 // 56 k walks at bounce 4 of a 1080p frame: 1.547 -> 1.510 ms for the frame, its two-level form 1.608 -> 1.585, four 720p
-// frames 2.242 -> 2.187); in the grids of small images, sized to their queues, groups of two are.
+// frames 2.242 -> 2.187); in the grids of small images, sized to their queues, groups of two are.  Where between
+// those the two measure alike is not known.
 constexpr uint32_t kPairMaxWalks = 1u << 15;
 
 // SHARE only sets the two kernels' copies apart: ptxas 13.0 crashes on one function called by both.

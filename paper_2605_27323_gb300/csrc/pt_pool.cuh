@@ -8,15 +8,17 @@
 //   - node steps repeat while at least kNodeLanes lanes hold an inner node;
 //   - then all lanes that hold a leaf test it together;
 //   - once kIdleLanes lanes have finished, they write their results and take the next slots.
-// Extension (closest-hit) and shadow (any-hit) rays share the loop, so a launch drains its warps once
-// and not once per kind.  Each ray visits the nodes and triangles of the lockstep walk in the same
-// order, so hits are the same bit for bit.
+// (Persistent warps that refill idle lanes from a pool of rays: Aila and Laine, "Understanding the Efficiency of Ray
+// Traversal on GPUs", HPG 2009.)  Extension (closest-hit) and shadow (any-hit) rays share the loop, so a launch drains
+// its warps once and not once per kind.  Each ray visits the nodes and triangles of the lockstep walk in the same
+// order, so hits are the same bit for bit.  (The shared ends below, and the groups of lanes of launches with few walks,
+// visit some more: subtrees walked before another lane's hit culls them.  Their hits are the same too.)
 //
-// What bounds it, in the launch of bounce 1 at 1080p on 1.15 M triangles: the L1 data path, busy 78% of the time with
+// What bounds it, in the launch of bounce 1 at 1080p on 1.15 M triangles: the L1 data path, busy 82% of the time with
 // divergent node requests (issue 61%, long-scoreboard stalls for the rest).  Requests fill it, not bytes: a node as
 // two 256-bit loads beats four of 128 bits by 1%, and reading its 56 used bytes in three loads costs 2% on the
-// terrain.  Against the lockstep walk: 168 -> 114 warp instructions per walk, 9.5 -> 18 lanes per instruction, 683
-// -> 531 us; camera rays 117 -> 91, 15 -> 23, 360 -> 282 us.
+// terrain.  Against the lockstep walk: 168 -> 115 warp instructions per walk, 9.5 -> 19 lanes per instruction, 683
+// -> 524 us; camera rays 117 -> 92, 15 -> 23, 360 -> 275 us.
 #pragma once
 #include "pt_common.cuh"
 
@@ -24,10 +26,10 @@ namespace pt {
 
 constexpr uint32_t kDone = 0xFFFFFFFFu;    // no subtree left (never a leaf reference: triangles < 2^28)
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
-// 8 and 20 measured best over the frames of {8, 10, 12} x {8, 12, 16, 20} lanes (1080p 1.600 ms against 1.648 at
-// 12 and 12, 1.658 at 12 and 8; the terrain 9.61 against 9.87 and 10.18): fewer node lanes waste L1 cycles, more
-// make the loop leave its node steps too often; a refill costs some 150 instructions and a claim for the
-// whole warp, however few lanes it serves.
+// 8 and 20 measured best over the frames of {8, 10, 12} x {8, 12, 16, 20} lanes; they are the lowest and the highest
+// tried, and were tried before the last walks were shared (1080p 1.600 ms against 1.648 at 12 and 12, 1.658 at 12 and
+// 8; the terrain 9.61 against 9.87 and 10.18): fewer node lanes waste L1 cycles, more make the loop leave its node steps
+// too often; a refill costs some 150 instructions and a claim for the whole warp, however few lanes it serves.
 constexpr uint32_t kNodeLanes = 8;
 constexpr uint32_t kIdleLanes = 20;
 // Fault guards against trees that the builder refuses (deeper than the stack) or never makes (cycles).  A phase takes at
@@ -212,7 +214,8 @@ constexpr uint32_t kAnySlot = 0x80000000u;
 
 // The end of a pool.  With no slot left, lanes run dry while the longest walks -- chains of several hundred
 // dependent node loads -- keep the launch alive.  Here the walks that are left belong to the warp: a lane
-// without work takes the oldest deferred subtree (the one nearest the root) of a lane that holds one, with
+// without work takes the oldest deferred subtree (the one nearest the root; as in work stealing, Blumofe and Leiserson,
+// "Scheduling Multithreaded Computations by Work Stealing", 1999) of a lane that holds one, with
 // that lane's ray, and walks it.  A ray's best hit so far, the smallest (t, original id), lies in shared memory under
 // its first lane's number; it culls every lane that works on the ray, and is the hit at the end: the closest-hit
 // rule makes it independent of the order of the walk (as in trace_closest_group).  When the slots ran out the
